@@ -1,8 +1,12 @@
 // Stiffness apply launchers and the per-voxel average stress; the kernels are in
-// apply_kernels.cuh.  This unit instantiates the one-interface kernels (two phases);
+// apply_kernels.cuh, apply_tile.cuh and apply_cut.cuh.  This unit instantiates the one-interface kernels (two phases);
 // apply_multi.cu instantiates those of two interfaces (three phases).
 #include "apply_kernels.cuh"
+#include "apply_tile.cuh"
 #include "apply_cut.cuh"
+
+#include <algorithm>
+#include <cmath>
 
 namespace xfft {
 
@@ -16,6 +20,53 @@ int apply_uncut_blocks(const GridDev& g) {
   const int gx = (g.n0 + kCX - 1) / kCX;
   return gz * gy * gx;
 }
+
+// Tile of the FP64 / double-word stencil.  The kernel is bound by the arithmetic pipe of its SMs,
+// so its time is about the operations of the busiest SM, in warp instructions: 210 per plane and
+// warp of voxels, 22 per plane and 32 of the tile's (ty + 1)(tz + 1) nodes (update, force sums), one
+// more node plane per item.  Items are cut small enough to spread evenly (a grid of 16^3 voxels is
+// 128 warps, one per SM); fewer than about four warps per SM leave the pipe waiting for its own
+// results.  Every tile shape that fills the block (equal parts of a row, as many rows as fit) and
+// power-of-two plane counts are compared by that estimate.
+TileShape pick_tile(const GridDev& g, int n_rhs) {
+  constexpr int kSMs = 152;
+  TileShape best = {};
+  double cost = 1e300;
+  for (int threads = 32; threads <= kTileThreads; threads *= 2)
+    for (int ntz = (g.n2 + threads - 1) / threads; ntz <= g.n2; ++ntz) {
+      const int tz = (g.n2 + ntz - 1) / ntz;
+      if (tz < 4 && tz < g.n2) break;
+      if ((g.n2 + tz - 1) / tz != ntz) continue;
+      int ty = std::min(threads / tz, g.n1);
+      const int nty = (g.n1 + ty - 1) / ty;
+      ty = (g.n1 + nty - 1) / nty;
+      if ((ty + 1) * (tz + 1) > 2 * kTileThreads) continue;
+      const int warps = (ty * tz + 31) / 32;
+      const double nodes = 22.0 * (((ty + 1) * (tz + 1) + 31) / 32);
+      for (int cx = 1; cx <= 16 && cx <= g.n0; cx *= 2) {
+        const int ncx = (g.n0 + cx - 1) / cx;
+        const double items = (double)nty * ntz * ncx * n_rhs;
+        const double per_sm = std::ceil(items / kSMs);  // items of the busiest SM
+        const double busy = std::min(1.0, per_sm * warps / 4.0);
+        const double c = per_sm * (cx * (210.0 * warps + nodes) + nodes) / busy;
+        if (c < cost * 0.999) {
+          cost = c;
+          best.threads = 32 * warps;
+          best.ty = ty;
+          best.tz = tz;
+          best.nty = nty;
+          best.ntz = ntz;
+          best.cx = cx;
+          best.ncx = ncx;
+        }
+      }
+    }
+  best.items = best.nty * best.ntz * best.ncx;
+  best.blocks = std::min(best.items, kTileMaxBlocks);
+  return best;
+}
+int apply_tile_blocks(const GridDev& g, int n_rhs) { return pick_tile(g, n_rhs).blocks; }
+int apply_tile_blocks_max() { return kTileMaxBlocks; }
 
 #ifndef XFFT_CUT_WAVES
 #define XFFT_CUT_WAVES 2
@@ -138,14 +189,15 @@ static cudaError_t launch_cut_cached(const float* d, float* q, CutData cd, const
 }
 
 // The enriched part of q only receives atomic contributions from the cut-tet kernel: it is
-// cleared first; the standard part must already hold the uncut kernel's plain stores.
+// cleared first (FP64, double-word: launch_apply_uncut has cleared all of q); the standard part
+// must already hold the uncut kernel's forces.
 template <typename T>
 cudaError_t launch_apply_cut(const typename Store<T>::type* d, typename Store<T>::type* q,
                              const typename Store<T>::type* isD, CutData cd, const ApplyArgs& a,
                              int n_rhs, cudaStream_t s) {
   typedef typename Store<T>::type S;
   const GridDev& g = a.g;
-  if (a.nX > 0) {
+  if (std::is_same<T, float>::value && a.nX > 0) {
     for (int r = 0; r < n_rhs; ++r) {
       cudaError_t e = cudaMemsetAsync(q + r * a.stride + 3 * g.N, 0, sizeof(S) * 3 * (size_t)a.nX, s);
       if (e != cudaSuccess) return e;

@@ -29,12 +29,6 @@ constexpr int kCX = XFFT_UNCUT_CX;  // output planes per block along x
 #ifndef XFFT_UNCUT_MINB
 #define XFFT_UNCUT_MINB 2  // resident blocks per SM asked of the FP32 uncut kernel
 #endif
-#ifndef XFFT_UNCUT_MINB64
-#define XFFT_UNCUT_MINB64 2  // resident blocks per SM asked of the FP64 uncut kernel
-#endif
-#ifndef XFFT_UNCUT_MINBDW
-#define XFFT_UNCUT_MINBDW 1  // resident blocks per SM asked of the double-word uncut kernel
-#endif
 
 template <typename T>
 __device__ __forceinline__ T cut_real(const CutData& cd, int f, int e);
@@ -282,9 +276,7 @@ __device__ __forceinline__ void edge_forces(const EdgeT<T>& te, T (&F)[8][3]) {
 #endif
 
 template <typename T, bool TOTAL, bool SIG, bool UNIFORM, bool FUSED, int NPH>
-__global__ void __launch_bounds__(kTZ* kTY, std::is_same<T, dw>::value     ? XFFT_UNCUT_MINBDW
-                                             : sizeof(T) == 8 ? XFFT_UNCUT_MINB64
-                                                              : XFFT_UNCUT_MINB)
+__global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
     k_apply_uncut(const typename Store<T>::type* __restrict__ d, typename Store<T>::type* __restrict__ q,
                   const ApplyArgs a, int nxchunks) {
   typedef typename Store<T>::type S;
@@ -551,52 +543,5 @@ __global__ void __launch_bounds__(kTZ* kTY, std::is_same<T, dw>::value     ? XFF
     for (int k = 0; k < 7; ++k) a.partials[((long long)rhs * 7 + k) * a.nparts + bid] = tot[k];
   }
 }
-
-// Stencil launches of one phase count NPH (2: one interface; 3: two interfaces).  The phase
-// counts are instantiated in separate translation units (apply.cu, apply_multi.cu).
-template <typename T, int NPH>
-cudaError_t launch_uncut_nph(const typename Store<T>::type* d, typename Store<T>::type* q,
-                             const ApplyArgs& a, int n_rhs, cudaStream_t s) {
-  const GridDev& g = a.g;
-  const int gz = (g.n2 + kTZ - 2) / (kTZ - 1);
-  const int gy = (g.n1 + kTY - 2) / (kTY - 1);
-  const int gx = (g.n0 + kCX - 1) / kCX;
-  dim3 block(kTZ, kTY, 1);
-  dim3 grid(gz, gy, gx * n_rhs);
-  const bool uni = g.h[0] == g.h[1] && g.h[1] == g.h[2];
-  const bool sig = a.want_sig || a.eps;
-#define XFFT_LAUNCH(TOT, SG, UNI) k_apply_uncut<T, TOT, SG, UNI, false, NPH><<<grid, block, 0, s>>>(d, q, a, gx)
-#define XFFT_LAUNCH_F(SG, UNI) k_apply_uncut<T, false, SG, UNI, true, NPH><<<grid, block, 0, s>>>(d, q, a, gx)
-  if (a.fz) {
-    // the fused CG update serves the FP32 and FP64 solvers (not the double-word residuals)
-    if constexpr (!std::is_same<T, dw>::value) {
-      if (sig) {
-        if (uni) XFFT_LAUNCH_F(true, true);
-        else XFFT_LAUNCH_F(true, false);
-      } else {
-        if (uni) XFFT_LAUNCH_F(false, true);
-        else XFFT_LAUNCH_F(false, false);
-      }
-    } else {
-      return cudaErrorInvalidValue;
-    }
-  } else if (a.eps) {
-    if (uni) XFFT_LAUNCH(true, true, true);
-    else XFFT_LAUNCH(true, true, false);
-  } else if (sig) {
-    if (uni) XFFT_LAUNCH(false, true, true);
-    else XFFT_LAUNCH(false, true, false);
-  } else {
-    if (uni) XFFT_LAUNCH(false, false, true);
-    else XFFT_LAUNCH(false, false, false);
-  }
-#undef XFFT_LAUNCH
-#undef XFFT_LAUNCH_F
-  return cudaGetLastError();
-}
-
-#define XFFT_APPLY_INST_NPH(EXT, T, NPH)                                                         \
-  EXT template cudaError_t launch_uncut_nph<T, NPH>(const Store<T>::type*, Store<T>::type*,      \
-                                                    const ApplyArgs&, int, cudaStream_t);
 
 }  // namespace xfft

@@ -1,6 +1,6 @@
 // Stiffness apply kernels of two interfaces (three phases, Sec. 4.2's coated sphere); the
 // one-interface kernels are instantiated in apply.cu.
-#include "apply_kernels.cuh"
+#include "apply_tile.cuh"
 
 namespace xfft {
 

@@ -653,6 +653,12 @@ static FinArgs fin_args(const xfft_ctx* c, int mode, int crit, double tol, int m
   return fa;
 }
 
+// slots of one partial-sum row: the widest of the kernels that write them
+static int nparts_of(const xfft_ctx* c) {
+  return std::max(std::max(apply_uncut_blocks(c->g), apply_tile_blocks_max()) + apply_cut_blocks_max(c->ncut),
+                  std::max(precondition_blocks(c->fft, c->nX, true), precondition_blocks(c->fft, c->nX, false)));
+}
+
 static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   const long long stride = stride_of(c);
   if (c->cap_rhs >= n_rhs && c->cap_stride == stride && c->cap_prec == prec) return XFFT_OK;
@@ -672,11 +678,8 @@ static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   CU(dalloc(c, &c->outer_mask, 64));
   CU(dalloc(c, &c->eps_d, 6 * 64));
   CU(dalloc(c, &c->sig_keep, 6 * 64));
-  const int na = apply_uncut_blocks(c->g) + apply_cut_blocks_max(c->ncut);
-  const int np =
-      std::max(precondition_blocks(c->fft, c->nX, true), precondition_blocks(c->fft, c->nX, false));
   const int ng = grad_blocks_uncut(c->g) + grad_blocks_cut(c->ncut);
-  const int nparts = std::max(na, np);
+  const int nparts = nparts_of(c);
   c->partials_count = std::max((size_t)n_rhs * 7 * nparts, (size_t)kGradValues * ng);
   CU(dalloc(c, &c->partials, c->partials_count));
   CU(dalloc(c, &c->red_out, 64));
@@ -693,9 +696,9 @@ static int cut_blocks_of(const xfft_ctx* c, bool fp32 = true) {
   return fp32 && c->cut_blocks > 0 ? c->cut_blocks : apply_cut_blocks(c->ncut);
 }
 
-static int nparts_of(const xfft_ctx* c) {
-  return std::max(apply_uncut_blocks(c->g) + apply_cut_blocks_max(c->ncut),
-                  std::max(precondition_blocks(c->fft, c->nX, true), precondition_blocks(c->fft, c->nX, false)));
+// partial-sum slots of the stencil (the cut-tet kernel's follow them)
+static int uncut_blocks_of(const xfft_ctx* c, bool fp32, int n_rhs) {
+  return fp32 ? apply_uncut_blocks(c->g) : apply_tile_blocks(c->g, n_rhs);
 }
 
 static ApplyArgs apply_args(const xfft_ctx* c, const double* eps, const int* active) {
@@ -768,7 +771,10 @@ static xfft_status do_apply(xfft_ctx* c, const T* d, T* q, const double* eps_dev
   const int kc = dwa ? XFFT_PROF_APPLY_CUT_DW : dbl ? XFFT_PROF_APPLY_CUT_F64 : XFFT_PROF_APPLY_CUT_F32;
   a.units_uncut = punit(c, ku);
   a.units_cut = punit(c, kc);
-  if (dbl || dwa) a.cut_blocks = a.cut_rpl = 0;  // the tuned shape is that of the FP32 kernel
+  if (dbl || dwa) {
+    a.cut_blocks = a.cut_rpl = 0;  // the tuned shape is that of the FP32 kernel
+    a.part_offset_cut = uncut_blocks_of(c, false, n_rhs);
+  }
   {
     ProfScope ps(c, ku, 1);
     CU(launch_apply_uncut<A>(d, q, a, n_rhs, c->stream));
@@ -779,7 +785,7 @@ static xfft_status do_apply(xfft_ctx* c, const T* d, T* q, const double* eps_dev
   }
   if (fin_mode >= 0) {
     FinArgs fa = fin_args(c, fin_mode, crit, tol, maxit, a.nparts,
-                          apply_uncut_blocks(c->g) + cut_blocks_of(c, !(dbl || dwa)), parity);
+                          a.part_offset_cut + cut_blocks_of(c, !(dbl || dwa)), parity);
     if (fin_mode == 0) {  // a residual phase: record its stress integrals (base of a later update)
       fa.sig_keep = c->sig_keep;
       fa.sig_base = sig_add ? c->sig_keep : nullptr;
@@ -1861,7 +1867,7 @@ static xfft_status apply_entry(xfft_ctx* c, int n_rhs, const double* d, const do
   if (st == XFFT_OK) st = stage_out<T>(c, qq, q, tot, on_dev, scratch);
   if (st == XFFT_OK && sigma_int) {
     const int nparts = nparts_of(c);
-    const int used = apply_uncut_blocks(c->g) + cut_blocks_of(c, sizeof(T) == 4);
+    const int used = uncut_blocks_of(c, sizeof(T) == 4, n_rhs) + cut_blocks_of(c, sizeof(T) == 4);
     cudaError_t e = launch_reduce_partials(c->partials, 7 * n_rhs, nparts, used, c->red_out, c->stream);
     double red[7 * 64];
     if (e == cudaSuccess)
@@ -2038,9 +2044,13 @@ extern "C" xfft_status xfft_apply_noalloc(xfft_ctx* c, int n_rhs, const double* 
   if (!c->have_micro) return fail(XFFT_ESTATE, "xfft_set_microstructure first");
   if (n_rhs < 1 || n_rhs > XFFT_NOALLOC_MAX_RHS)
     return fail(XFFT_EINVAL, "n_rhs must be in [1, XFFT_NOALLOC_MAX_RHS]");
-  const int nparts = apply_uncut_blocks(c->g) + apply_cut_blocks(c->ncut);
-  if (nparts > XFFT_NOALLOC_MAX_PARTS)
+  // the documented rule on the grid; the FP64 stencil's own blocks (at most apply_tile_blocks_max())
+  // and the cut-tet kernel's fit the scratch for every grid that it admits
+  if (apply_uncut_blocks(c->g) + apply_cut_blocks(c->ncut) > XFFT_NOALLOC_MAX_PARTS)
     return fail(XFFT_EINVAL, "grid too large for the fixed scratch of xfft_apply_noalloc");
+  const int tile_blocks = apply_tile_blocks(c->g, n_rhs);
+  const int nparts = tile_blocks + apply_cut_blocks(c->ncut);
+  if (nparts > XFFT_NOALLOC_MAX_PARTS) return fail(XFFT_EINVAL, "partial sums exceed the fixed scratch");
   double* scratch = nullptr;
   TRY(noalloc_scratch(&scratch, c->stream));
   ApplyArgs a;
@@ -2054,7 +2064,7 @@ extern "C" xfft_status xfft_apply_noalloc(xfft_ctx* c, int n_rhs, const double* 
   a.nX = c->nX;
   a.partials = scratch;
   a.nparts = nparts;
-  a.part_offset_cut = apply_uncut_blocks(c->g);
+  a.part_offset_cut = tile_blocks;
   a.units_uncut = nullptr;
   a.units_cut = nullptr;
   a.want_sig = 1;

@@ -132,6 +132,8 @@ template <typename T>
 cudaError_t launch_apply(const typename Store<T>::type* d, typename Store<T>::type* q,
                          const typename Store<T>::type* isD, CutData cd, const ApplyArgs& a,
                          int n_rhs, cudaStream_t s);
+// launch_apply_uncut writes the standard part of q; with FP64 or double-word arithmetic it clears
+// all of q first (n_rhs rows of a.stride)
 template <typename T>
 cudaError_t launch_apply_uncut(const typename Store<T>::type* d, typename Store<T>::type* q,
                                const ApplyArgs& a, int n_rhs, cudaStream_t s);
@@ -139,7 +141,9 @@ template <typename T>
 cudaError_t launch_apply_cut(const typename Store<T>::type* d, typename Store<T>::type* q,
                              const typename Store<T>::type* isD, CutData cd, const ApplyArgs& a,
                              int n_rhs, cudaStream_t s);
-int apply_uncut_blocks(const GridDev& g);
+int apply_uncut_blocks(const GridDev& g);               // FP32 stencil
+int apply_tile_blocks(const GridDev& g, int n_rhs);     // FP64 / double-word stencil
+int apply_tile_blocks_max();                            // the most it launches per right-hand side
 int apply_cut_blocks(int ncut);      // the default grid of the cut-tet kernel
 int apply_cut_blocks_max(int ncut);  // the largest grid a tuned launch shape may use
 
