@@ -347,7 +347,7 @@ extern "C" xfft_status xfft_create(xfft_ctx** out, const xfft_grid* grid, const 
   g.vol_tet = g.h[0] * g.h[1] * g.h[2] / 6.0;
   g.volY = grid->len[0] * grid->len[1] * grid->len[2];
   cudaError_t e = cudaSuccess;
-  c->fft = fft_plan_create(g, &e);
+  c->fft = fft_plan_create(g, o.precision == XFFT_FP64, &e);
   if (!c->fft || e != cudaSuccess) {
     delete c;
     return fail(XFFT_ECUDA, std::string("FFT plan: ") + cudaGetErrorString(e));
@@ -1901,6 +1901,7 @@ extern "C" xfft_status xfft_apply(xfft_ctx* c, int n_rhs, const double* d, const
 
 template <typename T>
 static xfft_status prec_entry(xfft_ctx* c, int n_rhs, const double* f, double* z, double* rr, int on_dev) {
+  CU(fft_plan_tables(c->fft, sizeof(T) == 8));
   const long long stride = stride_of(c);
   const size_t tot = (size_t)n_rhs * stride;
   double* scratch = nullptr;

@@ -277,55 +277,6 @@ struct Dft<C, 1, INV> {
   __host__ __device__ __forceinline__ static void run(C*) {}
 };
 
-// One in-place Stockham stage of radix R on a line (stride-1 elements at `line`), thread t of
-// the line's T = N / E threads.  NS = product of the previous radices.  tw[k] = exp(-2 pi i k/N).
-template <typename C, int N, int E, int R, int NS, bool INV>
-__device__ __forceinline__ void stage(C* line, const C* __restrict__ tw, int t) {
-  if (R == 1) return;
-  constexpr int T = N / E;
-  constexpr int NR = N / R;
-  constexpr int BPT = E / R;
-  C v[BPT][R];
-#pragma unroll
-  for (int b = 0; b < BPT; ++b) {
-    const int j = t + b * T;
-#pragma unroll
-    for (int r = 0; r < R; ++r) v[b][r] = line[j + r * NR];
-  }
-  __syncthreads();
-#pragma unroll
-  for (int b = 0; b < BPT; ++b) {
-    const int j = t + b * T;
-    const int jm = j % NS;
-    if (NS > 1) {
-      constexpr int step = N / (NS * R);
-#pragma unroll
-      for (int r = 1; r < R; ++r) {
-        const C w = tw[r * jm * step];
-        v[b][r] = INV ? cmulc(v[b][r], w) : cmul(v[b][r], w);
-      }
-    }
-    Dft<C, R, INV>::run(v[b]);
-    const int base = (j / NS) * NS * R + jm;
-#pragma unroll
-    for (int r = 0; r < R; ++r) line[base + r * NS] = v[b][r];
-  }
-  __syncthreads();
-}
-
-// Full line transform (all threads of the block must call it; t < N/E selects the thread's
-// position in its line, lines beyond the data may run on dummy storage).
-template <typename C, int N, bool INV>
-__device__ __forceinline__ void line_fft(C* line, const C* __restrict__ tw, int t) {
-  typedef Plan<N> P;
-  constexpr int E = P::E;
-  constexpr int N0 = 1, N1 = P::R0, N2 = P::R0 * P::R1, N3 = P::R0 * P::R1 * P::R2;
-  stage<C, N, E, P::R0, N0, INV>(line, tw, t);
-  stage<C, N, E, P::R1, N1, INV>(line, tw, t);
-  stage<C, N, E, P::R2, N2, INV>(line, tw, t);
-  stage<C, N, E, P::R3, N3, INV>(line, tw, t);
-}
-
 // ---------------------------------------------------------------- Green operator
 // Cholesky factor of M(xi) = (|T|/2) sum_tets (|G|^2 I + G G^H) (see fft.cu); returns false
 // at xi = 0 or on a non-positive pivot (the Green operator then maps to 0).  Host and device
@@ -420,12 +371,8 @@ __host__ __device__ __forceinline__ void green_solve(const GreenFactor<C, T>& gf
   F2 = x2;
 }
 
-// block: (k2, j), all three components of a group of rg right-hand sides: 3 rg contiguous lines
-// of length N = n0.  The symbol of each frequency is factorised once and applied to every
-// right-hand side of the group.
-
 // ---------------------------------------------------------------- lines with an address map
-// The same stages on a line whose element m lives at map.at(m) (any shared-memory layout; the
+// Stockham stages on a line whose element m lives at map.at(m) (any shared-memory layout; the
 // maps of different lines must be disjoint).  The first stage may read its inputs through a
 // different map `ld0` (ld0.get(m) returns the value).  Threads with act == false take part in
 // the barriers only.

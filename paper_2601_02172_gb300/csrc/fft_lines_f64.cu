@@ -1,0 +1,6 @@
+// Line passes of the preconditioner, FP64 instantiation (kernels in fft_lines.cuh).
+#include "fft_lines_launch.cuh"
+
+namespace xfft {
+XFFT_LINES_INST(double)
+}  // namespace xfft

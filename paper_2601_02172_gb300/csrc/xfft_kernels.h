@@ -153,7 +153,9 @@ cudaError_t launch_voxel_stress(const double* u, const double* isD, CutData cd,
 
 // ---- preconditioner (fft.cu)
 struct FftPlan;  // opaque
-FftPlan* fft_plan_create(const GridDev& g, cudaError_t* err);
+// the plan with the Green table of one precision (dbl: FP64); fft_plan_tables adds another's
+FftPlan* fft_plan_create(const GridDev& g, bool dbl, cudaError_t* err);
+cudaError_t fft_plan_tables(FftPlan* p, bool dbl);
 void fft_plan_destroy(FftPlan* p);
 size_t fft_spectrum_elems(const FftPlan* p);  // complex elements per RHS
 // z = P^-1 f per RHS (std part via FFT + Green, enr part identity); f^T z partials into
