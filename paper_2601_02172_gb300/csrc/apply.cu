@@ -4,6 +4,7 @@
 #include "apply_kernels.cuh"
 #include "apply_tile.cuh"
 #include "apply_cut.cuh"
+#include "apply_cut_el.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -83,6 +84,11 @@ int apply_cut_blocks_max(int ncut) {
   const int cap = nb < kCutBlocksTuneMax ? nb : kCutBlocksTuneMax;
   const int def = apply_cut_blocks(ncut);
   return cap > def ? cap : def;
+}
+
+int apply_cut_el_blocks(int ncut) {
+  const int nb = (ncut + 31) / 32;
+  return nb < 1 ? 1 : (nb > kElBlocksMax ? kElBlocksMax : nb);
 }
 
 template <typename T>
@@ -207,6 +213,15 @@ cudaError_t launch_apply_cut(const typename Store<T>::type* d, typename Store<T>
     if (a.kcache && !a.eps && !a.want_sig && cd.ncut > 0) return launch_cut_cached(d, q, cd, a, n_rhs, s);
   }
   // launched even without cut tets: its blocks write the (zero) partial sums of their slots
+  if constexpr (std::is_same<T, double>::value) {
+    if (cd.el) {
+      const int nb = apply_cut_el_blocks(cd.ncut) * n_rhs;
+      if (a.eps) k_apply_cut_el<true, true><<<nb, 32, 0, s>>>(d, q, cd, a, n_rhs);
+      else if (a.want_sig) k_apply_cut_el<false, true><<<nb, 32, 0, s>>>(d, q, cd, a, n_rhs);
+      else k_apply_cut_el<false, false><<<nb, 32, 0, s>>>(d, q, cd, a, n_rhs);
+      return cudaGetLastError();
+    }
+  }
   const int nb = a.cut_blocks > 0 ? a.cut_blocks : apply_cut_blocks(cd.ncut);
   const int rpl = a.cut_rpl > 0 && a.cut_rpl < kCutMaxR ? a.cut_rpl : kCutMaxR;
   const bool sig = a.want_sig || a.eps;

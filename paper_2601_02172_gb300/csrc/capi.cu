@@ -95,6 +95,7 @@ struct xfft_ctx {
   int4* cut_n4 = nullptr;
   int4* cut_e4 = nullptr;
   double* cut_r64 = nullptr;
+  double* cut_el = nullptr;  // reduced element records (FP64 solvers)
   float* cut_r32 = nullptr;
   double* D = nullptr;
   double* isD = nullptr;
@@ -251,6 +252,7 @@ static CutData cutdata(const xfft_ctx* c) {
   cd.n4 = c->cut_n4;
   cd.e4 = c->cut_e4;
   cd.r64 = c->cut_r64;
+  cd.el = c->cut_el;
   cd.r32 = c->cut_r32;
   return cd;
 }
@@ -400,6 +402,7 @@ static void free_micro(xfft_ctx* c) {
   dfree(c, c->cut_n4);
   dfree(c, c->cut_e4);
   dfree(c, c->cut_r64);
+  dfree(c, c->cut_el);
   dfree(c, c->cut_r32);
   dfree(c, c->D);
   dfree(c, c->isD);
@@ -609,6 +612,15 @@ extern "C" xfft_status xfft_set_microstructure_phases(xfft_ctx* c, int n_levelse
   CU(dalloc(c, &c->cut_r32, (size_t)kRec * c->ncut));
   CU(launch_cut_records(cd, c->isD, c->nX, g, c->ph, c->has_scale ? c->scale : nullptr, c->cut_n4,
                         c->cut_e4, c->cut_r64, c->cut_r32, s));
+  if (c->opt.precision == XFFT_FP64 && c->ncut > 0) {
+    // 1 KB per cut tet; where it does not fit (max_device_bytes, device memory) the FP64 applies run
+    // on the moment records, with more arithmetic
+    const cudaError_t ea = dalloc(c, &c->cut_el, cut_el_reals(c->ncut));
+    if (ea == cudaSuccess)
+      CU(launch_cut_elements(cd, c->isD, c->nX, g, c->ph, c->has_scale ? c->scale : nullptr, c->cut_el, s));
+    else
+      cudaGetLastError();
+  }
   if (c->opt.precision == XFFT_FP32_REFINED && c->opt.cut_cache && c->ncut > 0) {
     CU(dalloc(c, &c->kcache, (size_t)kCutPacked * c->ncut));
     CU(launch_cut_matrix(cd, c->isD, c->nX, g, c->ph, c->has_scale ? c->scale : nullptr, c->kcache, s));
@@ -655,7 +667,8 @@ static FinArgs fin_args(const xfft_ctx* c, int mode, int crit, double tol, int m
 
 // slots of one partial-sum row: the widest of the kernels that write them
 static int nparts_of(const xfft_ctx* c) {
-  return std::max(std::max(apply_uncut_blocks(c->g), apply_tile_blocks_max()) + apply_cut_blocks_max(c->ncut),
+  return std::max(std::max(apply_uncut_blocks(c->g), apply_tile_blocks_max()) +
+                      std::max(apply_cut_blocks_max(c->ncut), apply_cut_el_blocks(c->ncut)),
                   std::max(precondition_blocks(c->fft, c->nX, true), precondition_blocks(c->fft, c->nX, false)));
 }
 
@@ -690,9 +703,10 @@ static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   return XFFT_OK;
 }
 
-// the cut-tet kernel's grid of a launch (its partial slots are reserved for the largest tuned
-// grid): the tuned grid for the FP32 kernel, the default for the FP64 and double-word kernels
-static int cut_blocks_of(const xfft_ctx* c, bool fp32 = true) {
+// the cut-tet kernel's grid of a launch (its partial slots are reserved for the largest grid): the
+// tuned grid for the FP32 kernel, the reduced records' for FP64 where they exist, else the default
+static int cut_blocks_of(const xfft_ctx* c, bool fp32 = true, bool dwa = false) {
+  if (!fp32 && !dwa && c->cut_el) return apply_cut_el_blocks(c->ncut);
   return fp32 && c->cut_blocks > 0 ? c->cut_blocks : apply_cut_blocks(c->ncut);
 }
 
@@ -785,7 +799,7 @@ static xfft_status do_apply(xfft_ctx* c, const T* d, T* q, const double* eps_dev
   }
   if (fin_mode >= 0) {
     FinArgs fa = fin_args(c, fin_mode, crit, tol, maxit, a.nparts,
-                          a.part_offset_cut + cut_blocks_of(c, !(dbl || dwa)), parity);
+                          a.part_offset_cut + cut_blocks_of(c, !(dbl || dwa), dwa), parity);
     if (fin_mode == 0) {  // a residual phase: record its stress integrals (base of a later update)
       fa.sig_keep = c->sig_keep;
       fa.sig_base = sig_add ? c->sig_keep : nullptr;
@@ -1867,7 +1881,7 @@ static xfft_status apply_entry(xfft_ctx* c, int n_rhs, const double* d, const do
   if (st == XFFT_OK) st = stage_out<T>(c, qq, q, tot, on_dev, scratch);
   if (st == XFFT_OK && sigma_int) {
     const int nparts = nparts_of(c);
-    const int used = uncut_blocks_of(c, sizeof(T) == 4, n_rhs) + cut_blocks_of(c, sizeof(T) == 4);
+    const int used = uncut_blocks_of(c, sizeof(T) == 4, n_rhs) + cut_blocks_of(c, sizeof(T) == 4, std::is_same<A, dw>::value);
     cudaError_t e = launch_reduce_partials(c->partials, 7 * n_rhs, nparts, used, c->red_out, c->stream);
     double red[7 * 64];
     if (e == cudaSuccess)
@@ -2050,7 +2064,7 @@ extern "C" xfft_status xfft_apply_noalloc(xfft_ctx* c, int n_rhs, const double* 
   if (apply_uncut_blocks(c->g) + apply_cut_blocks(c->ncut) > XFFT_NOALLOC_MAX_PARTS)
     return fail(XFFT_EINVAL, "grid too large for the fixed scratch of xfft_apply_noalloc");
   const int tile_blocks = apply_tile_blocks(c->g, n_rhs);
-  const int nparts = tile_blocks + apply_cut_blocks(c->ncut);
+  const int nparts = tile_blocks + cut_blocks_of(c, false);
   if (nparts > XFFT_NOALLOC_MAX_PARTS) return fail(XFFT_EINVAL, "partial sums exceed the fixed scratch");
   double* scratch = nullptr;
   TRY(noalloc_scratch(&scratch, c->stream));

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "apply_cut_el.cuh"
 #include "cut_geometry.cuh"
 #include "xfft_kernels.h"
 
@@ -485,6 +486,66 @@ __global__ void k_cut_matrix(const int* __restrict__ ip, const double* __restric
     for (int i = 0; i < 24; ++i)
       for (int j = i; j < 24; ++j, ++k) kc[(long long)k * ncut + e] = (float)cut_element_entry(i, j, w, gr, dsc);
   }
+}
+
+// Reduced element records (apply_cut_el.cuh): with D0^-1/2 = dsc folded in, l_b and p_b / 2 from
+// v_sb = (m.c)_s g_b + m_sb gamma_s, the enriched block from the cached-matrix entries.
+__global__ void __launch_bounds__(128) k_cut_elements(const int* __restrict__ ip, const double* __restrict__ dp,
+                                                      const double* __restrict__ isD, int nX, int ncut, GridDev g,
+                                                      PhaseDev ph, const float* __restrict__ scale,
+                                                      double* __restrict__ el) {
+  const double ih[3] = {1.0 / g.h[0], 1.0 / g.h[1], 1.0 / g.h[2]};
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ncut; e += gridDim.x * blockDim.x) {
+    const int vox = ip[8 * ncut + e];
+    const int t = ip[9 * ncut + e];
+    const int sph = ip[kCutFieldPhases * ncut + e];
+    double gr[4][3];
+    tet_grads<double>(t, ih, gr);
+    double L[4], dsc[4][3];
+    for (int a = 0; a < 4; ++a) {
+      L[a] = dp[(long long)cut_f_L(a) * ncut + e];
+      const int j = ip[(4 + a) * ncut + e];
+      for (int x = 0; x < 3; ++x) dsc[a][x] = isD[(long long)x * nX + j];
+    }
+    const double sv = scale ? (double)scale[vox] : 1.0;
+    SideW w[2];
+    double lam = 0.0, mu = 0.0, l[4][3] = {}, p[4][3] = {};
+    for (int si = 0; si < 2; ++si) {
+      const int f = si == 0 ? cut_phase_plus(sph) : cut_phase_minus(sph);
+      double Mp[10];
+      for (int k = 0; k < 10; ++k) Mp[k] = dp[(long long)cut_f_M(si, k) * ncut + e];
+      side_weights(L, si == 0 ? 1.0 : -1.0, gr, Mp, ph.lam[f] * sv, ph.mu[f] * sv, w[si]);
+      const SideW& W = w[si];
+      lam += W.V * W.lam;
+      mu += W.V * W.mu;
+      for (int b = 0; b < 4; ++b)
+        for (int x = 0; x < 3; ++x) {
+          const double v = W.P * gr[b][x] + W.m[b] * W.gam[x];
+          l[b][x] += W.lam * v;
+          p[b][x] += W.mu * v;
+        }
+    }
+    double* R = el + ((long long)(e >> 5) * kEl) * 32 + (e & 31);
+    R[0] = lam;
+    R[32] = mu;
+    for (int b = 0; b < 4; ++b)
+      for (int x = 0; x < 3; ++x) {
+        R[32 * (kElL + 3 * b + x)] = dsc[b][x] * l[b][x];
+        for (int y = 0; y < 3; ++y) R[32 * (kElP + 9 * b + 3 * x + y)] = dsc[b][x] * p[b][y];
+      }
+    int k = 0;
+    for (int i = 0; i < 12; ++i)
+      for (int j = i; j < 12; ++j, ++k) R[32 * (kElK + k)] = cut_element_entry(12 + i, 12 + j, w, gr, dsc);
+  }
+}
+
+size_t cut_el_reals(int ncut) { return (size_t)((ncut + 31) / 32) * 32 * kEl; }
+
+cudaError_t launch_cut_elements(CutData cd, const double* isD, int nX, GridDev g, PhaseDev ph,
+                                const float* scale, double* el, cudaStream_t s) {
+  if (cd.ncut == 0) return cudaSuccess;
+  k_cut_elements<<<(cd.ncut + 127) / 128, 128, 0, s>>>(cd.ip, cd.dp, isD, nX, cd.ncut, g, ph, scale, el);
+  return cudaGetLastError();
 }
 
 __global__ void k_cut_records(const int* __restrict__ ip, const double* __restrict__ dp,

@@ -29,6 +29,8 @@ struct CutData {
   const int4* e4 = nullptr;
   const float* r32 = nullptr;
   const double* r64 = nullptr;
+  // FP64 solvers: reduced element records of apply_cut_el.cuh (groups of 32 tets)
+  const double* el = nullptr;
 };
 // Apply record of a cut tet (tet-major, kRec reals, 16-byte aligned groups):
 //   [3a + c]            D0^-1/2 of the enriched DOF (vertex a, component c)
@@ -91,6 +93,10 @@ cudaError_t launch_cut_records(CutData cd, const double* isD, int nX, GridDev g,
                                cudaStream_t s);
 // cached scaled element matrices of the cut tets (packed upper triangle, FP32; isD: D0^-1/2)
 constexpr int kCutPacked = 24 * 25 / 2;
+// reduced element records of the FP64 solvers (layout in apply_cut_el.cuh): cut_el_reals(ncut) doubles
+size_t cut_el_reals(int ncut);
+cudaError_t launch_cut_elements(CutData cd, const double* isD, int nX, GridDev g, PhaseDev ph,
+                                const float* scale, double* el, cudaStream_t s);
 cudaError_t launch_cut_matrix(CutData cd, const double* isD, int nX, GridDev g, PhaseDev ph,
                               const float* scale, float* kc, cudaStream_t s);
 
@@ -146,6 +152,7 @@ int apply_tile_blocks(const GridDev& g, int n_rhs);     // FP64 / double-word st
 int apply_tile_blocks_max();                            // the most it launches per right-hand side
 int apply_cut_blocks(int ncut);      // the default grid of the cut-tet kernel
 int apply_cut_blocks_max(int ncut);  // the largest grid a tuned launch shape may use
+int apply_cut_el_blocks(int ncut);   // the grid of the FP64 kernel on reduced records
 
 // per-voxel average stress of the (scaled) solution u, double
 cudaError_t launch_voxel_stress(const double* u, const double* isD, CutData cd,
