@@ -67,7 +67,7 @@ __device__ __forceinline__ void tile_tet(const T (&D)[12][3], T (&Te)[12][3], T 
 }
 
 template <typename T, bool TOTAL, bool SIG, bool UNIFORM, bool FUSED, int NPH>
-__global__ void __launch_bounds__(kTileThreads, 2)
+__global__ void __launch_bounds__(kTileThreads, 3)
     k_apply_tile(const typename Store<T>::type* __restrict__ d, typename Store<T>::type* __restrict__ q,
                  const ApplyArgs a, const TileShape ts) {
   typedef typename Store<T>::type S;
