@@ -535,8 +535,13 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
   const double r2 = 1.41421356237309504880;
   double v[7] = {to_double(en), to_double(sg[0]), to_double(sg[1]), to_double(sg[2]),
                  to_double(sg[3]) * r2, to_double(sg[4]) * r2, to_double(sg[5]) * r2};
-  double tot[7];
-  block_sum<7>(v, red, tot);
+  double tot[7] = {};
+  if (SIG) {
+    block_sum<7>(v, red, tot);
+  } else {
+    __shared__ T red1[kTZ * kTY];
+    tot[0] = block_sum1<T>(en, red1);
+  }
   if (tid == 0) {
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * xc);
 #pragma unroll

@@ -238,8 +238,13 @@ __global__ void k_finalize(RhsState* __restrict__ st, int* __restrict__ act,
   double v[7] = {0, 0, 0, 0, 0, 0, 0};
   for (int i = threadIdx.x; i < ncount; i += blockDim.x)
     for (int k = 0; k < nread; ++k) v[k] += partials[((long long)rhs * nv + k) * fa.nparts + i];
-  double tot[7];
-  block_sum<7>(v, red, tot);
+  double tot[7] = {};
+  if (nread == 1) {
+    __shared__ double red1[512];
+    tot[0] = block_sum1<double>(v[0], red1);
+  } else {
+    block_sum<7>(v, red, tot);
+  }
   if (threadIdx.x != 0) return;
   if (fa.mode == 0) {
     for (int k = 0; k < 6; ++k) s.sig[k] = (fa.sig_base ? fa.sig_base[6 * rhs + k] : 0.0) + tot[1 + k];

@@ -63,7 +63,7 @@ __global__ void k_enr_precond(T* __restrict__ f, T* __restrict__ z, long long st
                               double* __restrict__ partials, int nparts, int slot0,
                               const T* __restrict__ q, const RhsState* __restrict__ st,
                               const T* __restrict__ eblk) {
-  __shared__ double red[32];
+  __shared__ T red[256];
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) return;
   T* fr = f + rhs * stride + off;
@@ -106,9 +106,8 @@ __global__ void k_enr_precond(T* __restrict__ f, T* __restrict__ z, long long st
       acc += v[0] * z0 + v[1] * z1 + v[2] * z2;
     }
   }
-  double vv[1] = {(double)acc}, tot[1];
-  block_sum<1>(vv, red, tot);
-  if (threadIdx.x == 0) partials[(long long)rhs * nparts + slot0 + blockIdx.x] = tot[0];
+  const double tot = block_sum1<T>(acc, red);
+  if (threadIdx.x == 0) partials[(long long)rhs * nparts + slot0 + blockIdx.x] = tot;
 }
 
 // ---------------------------------------------------------------- plan

@@ -497,7 +497,7 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR>())
                  double* __restrict__ partials, int nparts) {
   typedef typename CplxOf<T>::type C;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ double red[32];
+  __shared__ T red[kLineThreads];
   const int rhs = blockIdx.y;
   if (active && !active[rhs]) return;
   C* buf = reinterpret_cast<C*>(smraw);
@@ -600,9 +600,8 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR>())
       acc += a.y * g[r].y;
     }
   });
-  double vv[1] = {(double)acc}, tot[1];
-  block_sum<1>(vv, red, tot);
-  if (threadIdx.x == 0) partials[(long long)rhs * nparts + blockIdx.x] = tot[0];
+  const double tot = block_sum1<T>(acc, red);
+  if (threadIdx.x == 0) partials[(long long)rhs * nparts + blockIdx.x] = tot;
 }
 
 // ---------------------------------------------------------------- Green table

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(Sq<N>::NT, Sq<N>::MINB) ks_inv(const float2* _
   constexpr int N1 = Sq<N>::N1, N2 = Sq<N>::N2, H2 = Sq<N>::H2, PL = Sq<N>::PL, RS = Sq<N>::RS;
   constexpr int E = Sq<N>::E, NT = Sq<N>::NT;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ double red[32];
+  __shared__ float red[NT];
   float2* tws1 = reinterpret_cast<float2*>(smraw);
   float2* tws2 = tws1 + N1;
   float2* buf = tws2 + N2;
@@ -269,9 +269,8 @@ __global__ void __launch_bounds__(Sq<N>::NT, Sq<N>::MINB) ks_inv(const float2* _
       acc += val * fv[e];
     }
   }
-  double vv[1] = {(double)acc}, tot[1];
-  block_sum<1>(vv, red, tot);
-  if (threadIdx.x == 0) partials[(long long)rhs * nparts + blockIdx.x] = tot[0];
+  const double tot = block_sum1<float>(acc, red);
+  if (threadIdx.x == 0) partials[(long long)rhs * nparts + blockIdx.x] = tot;
 }
 
 // ---------------------------------------------------------------- Green factor table

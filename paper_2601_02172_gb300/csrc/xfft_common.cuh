@@ -90,6 +90,33 @@ __device__ inline T warp_sum(T v) {
   return v;
 }
 
+// The reductions below count FP64 additions: the SM issues one warp-wide FP64 instruction every 16
+// clocks, so seven butterfly sums of five steps in each of eight warps hold its pipe for 5000 clocks
+// per block (a tenth of the FP32 stencil's time at 128^3, 15 us of every finalisation).
+
+// Sums of eight values over a warp in nine additions instead of 40: each of the first three steps
+// halves the number of values a lane carries.  Lane l returns the total of v[l / 4].
+__device__ inline double warp_sum8(const double (&v)[8]) {
+  const int lane = (threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z)) & 31;
+  double w4[4], w2[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const bool hi = lane & 16;
+    const double other = __shfl_xor_sync(0xffffffffu, hi ? v[i] : v[i + 4], 16);
+    w4[i] = (hi ? v[i + 4] : v[i]) + other;
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const bool hi = lane & 8;
+    const double other = __shfl_xor_sync(0xffffffffu, hi ? w4[i] : w4[i + 2], 8);
+    w2[i] = (hi ? w4[i + 2] : w4[i]) + other;
+  }
+  const bool hi = lane & 4;
+  double w = (hi ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, hi ? w2[0] : w2[1], 4);
+  w += __shfl_xor_sync(0xffffffffu, w, 2);
+  return w + __shfl_xor_sync(0xffffffffu, w, 1);
+}
+
 // Sum NV values over the block (any 1D/2D/3D shape, a multiple of 32 threads); thread 0
 // receives the totals in out[].  smem must hold NV * 32 doubles.  All threads must call it.
 template <int NV>
@@ -97,22 +124,54 @@ __device__ inline void block_sum(const double (&v)[NV], double* smem, double (&o
   const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
   const int nw = (blockDim.x * blockDim.y * blockDim.z) >> 5;
   const int lane = tid & 31, wid = tid >> 5;
-  double w[NV];
+  if constexpr (NV > 2 && NV <= 8) {
+    double w[8];
 #pragma unroll
-  for (int i = 0; i < NV; ++i) w[i] = warp_sum(v[i]);
-  if (lane == 0) {
+    for (int i = 0; i < 8; ++i) w[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
+    const double s = warp_sum8(w);
+    if ((lane & 3) == 0 && lane / 4 < NV) smem[(lane / 4) * 32 + wid] = s;
+    __syncthreads();
+    if (wid == 0) {  // lane i adds value i over the warps, in their order
+      double t = 0.0;
+      if (lane < NV)
+        for (int k = 0; k < nw; ++k) t += smem[lane * 32 + k];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) smem[i * 32 + wid] = w[i];
-  }
-  __syncthreads();
-  if (wid == 0) {
+      for (int i = 0; i < NV; ++i) out[i] = __shfl_sync(0xffffffffu, t, i);
+    }
+  } else {
+    double w[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      double s = lane < nw ? smem[i * 32 + lane] : 0.0;
-      out[i] = warp_sum(s);
+    for (int i = 0; i < NV; ++i) w[i] = warp_sum(v[i]);
+    if (lane == 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) smem[i * 32 + wid] = w[i];
+    }
+    __syncthreads();
+    if (wid == 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) {
+        double s = lane < nw ? smem[i * 32 + lane] : 0.0;
+        out[i] = warp_sum(s);
+      }
     }
   }
   __syncthreads();
+}
+
+// Sum of one value per thread over the block, in FP64 by its first warp (threads / 32 + 5 additions);
+// every thread of that warp receives it.  smem: one T per thread.  All threads must call it.
+template <typename T>
+__device__ inline double block_sum1(T v, T* smem) {
+  const int tid = threadIdx.x + blockDim.x * (threadIdx.y + blockDim.y * threadIdx.z);
+  const int n = blockDim.x * blockDim.y * blockDim.z;
+  smem[tid] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (tid < 32) {
+    for (int i = tid; i < n; i += 32) s += (double)smem[i];
+    s = warp_sum(s);
+  }
+  return s;
 }
 
 // Per-RHS solver state, FP64 scalars (Algorithm 1).
