@@ -2,11 +2,9 @@
 //   q = sum_e Lambda_e^T int_e B~^T C (eps_bar + B~ d_e)        (eps_bar only in TOTAL mode)
 // with fused reductions <d, A d> = sum_e int eps(d) : C : eps(d) and int_Y C (eps_bar + grad^s d).
 //
-// Uncut tets (constant strain, one phase): a 2.5-D marching kernel.  A block of kTZ x kTY
-// (16 x 16) threads owns one voxel column each (y, z) and walks along x; node planes of d are
-// staged in shared memory, each voxel's six Kuhn tets are evaluated once, the 8 corner forces are
-// combined along z by warp shuffles and along y through shared memory, and the x direction is
-// carried in registers, so every node force is written exactly once with a plain store.
+// Uncut tets (constant strain, one phase): the FP32 kernel here marches along x in 2.5 D, the FP64
+// and double-word one is apply_tile.cuh; both evaluate a voxel's six Kuhn tets by its edges (cube_edge,
+// voxel_tet below).
 //
 // Cut tets: apply_cut.cuh (one thread per cut tet, atomics after the uncut kernel).
 #pragma once
@@ -134,152 +132,129 @@ __device__ __forceinline__ void tet_uncut(const T (&u)[8][3], T (&F)[8][3], unsi
 }
 
 // ---------------------------------------------------------------- uncut stencil
-// Node values staged in shared memory as 4-vectors (one 16- or 32-byte load per corner).
-template <typename T>
-struct Node4 {
-  T x, y, z, w;
-};
-template <typename T>
-__device__ __forceinline__ T comp(const Node4<T>& v, int i) {
-  return i == 0 ? v.x : (i == 1 ? v.y : v.z);
+// edge of the cube along axis k starting at corner c (bit k of c is 0): 4 k + the other two bits
+__host__ __device__ constexpr int cube_edge(int c, int k) {
+  return 4 * k + (k == 0 ? c >> 1 : k == 1 ? (c & 1) | ((c >> 2) << 1) : c & 3);
 }
 
-// Per-voxel coefficients of the uncut tets, per phase ph (one interface: 0 minus, 1 plus; NPH
-// phases in all) and axis k:
-//   lw[ph][k] = lambda w_k s_v, mw[ph][k] = mu w_k s_v with w_k = |T| / h_k^2 on a uniform grid
-//   (raw node differences) or |T| / h_k otherwise (differences scaled by 1/h_k).
-template <typename T, bool UNIFORM, int NPH>
-struct Coef {
-  T lw[NPH][UNIFORM ? 1 : 3];
-  T mw[NPH][UNIFORM ? 1 : 3];
-  __device__ __forceinline__ T l(int ph, int k) const { return lw[ph][UNIFORM ? 0 : k]; }
-  __device__ __forceinline__ T m(int ph, int k) const { return mw[ph][UNIFORM ? 0 : k]; }
-};
-
-// One uncut Kuhn tet: the displacement-gradient columns of the tet are the node differences
-// along its path 0 -> e_p -> e_p+e_q -> (1,1,1); the edge tensions T_k = w_k sigma e_k move
-// the corner forces: F[0] -= T_p, F[c1] += T_p - T_q, F[c2] += T_q - T_r, F[7] += T_r.
-// Edge tensions of a voxel, summed over its tets: first edges 0 -> e_p (TE0[p]), middle edges
-// e_p -> e_p + e_q (TEM[p][q]), last edges e_p + e_q -> (1,1,1) (TEL[r], r the third axis).
-template <typename T>
-struct EdgeT {
-  T e0[3][3], em[3][3][3], el[3][3];
-};
-
-// EDGE: add the tet's tensions to the voxel's edge sums (corner forces formed once per voxel by
-// edge_forces); otherwise add them to the corner forces F directly.
-template <typename T, int t, bool TOTAL, bool SIG, bool UNIFORM, int NPH, bool EDGE = false>
-__device__ __forceinline__ void tet_stencil(const Node4<T> (&u)[8], T (&F)[8][3], unsigned code,
-                                            const Coef<T, UNIFORM, NPH>& cf, const T (&ih)[3],
-                                            const T (&hk)[3], const T (&Eb)[3][3], T& en, T (&sg)[6],
-                                            EdgeT<T>* te = nullptr) {
+// One Kuhn tet: the displacement-gradient columns of the tet are the node differences D along its
+// path 0 -> e_p -> e_p+e_q -> (1,1,1); its tensions sigma e_k are added to (or, as the edge's first
+// contribution, stored in) the voxel's edge sums Te.  l, m: lambda, mu of the tet (zero for a cut
+// tet) times the voxel scale.
+template <typename T, int t>
+__device__ __forceinline__ void voxel_tet(const T (&D)[12][3], T (&Te)[12][3], T l, T m) {
   constexpr int p = perm_p(t), q = perm_q(t), r = perm_r(t);
-  constexpr int c1 = tet_c1(t), c2 = tet_c2(t);
-  const unsigned cd = (code >> (2 * t)) & 3u;
-  if (cd == kCodeCut) return;
-  const int ph = NPH == 2 ? (int)cd : code_phase(cd);
-  T G[3][3];  // G[k][i]: column k (axis k) of the gradient, component i
+  constexpr int E[3] = {p == 0 ? cube_edge(0, 0) : q == 0 ? cube_edge(1 << p, 0) : cube_edge(6, 0),
+                        p == 1 ? cube_edge(0, 1) : q == 1 ? cube_edge(1 << p, 1) : cube_edge(5, 1),
+                        p == 2 ? cube_edge(0, 2) : q == 2 ? cube_edge(1 << p, 2) : cube_edge(3, 2)};
+  // the first tet that reaches a shared edge stores; p edges are shared by tets 2p and 2p + 1
+  constexpr bool first_r = t == 0 || t == 1 || t == 3;
+  const T tr = D[E[0]][0] + D[E[1]][1] + D[E[2]][2];
+  const T s01 = D[E[0]][1] + D[E[1]][0], s02 = D[E[0]][2] + D[E[2]][0], s12 = D[E[1]][2] + D[E[2]][1];
+  const T m2 = m + m;
+  const T lt = l * tr;
+  const T t01 = m * s01, t02 = m * s02, t12 = m * s12;
+  // sigma of the tet (times the common factor of l and m): column k is its tension on the edge
+  // along k, up to the weight w_k that the corner forces apply
+  const T S[3][3] = {{lt + m2 * D[E[0]][0], t01, t02}, {t01, lt + m2 * D[E[1]][1], t12}, {t02, t12, lt + m2 * D[E[2]][2]}};
 #pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    G[p][i] = comp(u[c1], i) - comp(u[0], i);
-    G[q][i] = comp(u[c2], i) - comp(u[c1], i);
-    G[r][i] = comp(u[7], i) - comp(u[c2], i);
-  }
-  if (!UNIFORM) {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      G[0][i] *= ih[0];
-      G[1][i] *= ih[1];
-      G[2][i] *= ih[2];
-    }
-  }
-  T Dr[3][3];  // unmodified columns for the energy
-  if (SIG) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) Dr[k][i] = G[k][i];
-  }
-  if (TOTAL) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) G[k][i] += Eb[i][k];
-  }
-  const T tr = G[0][0] + G[1][1] + G[2][2];
-  const T s01 = G[0][1] + G[1][0], s02 = G[0][2] + G[2][0], s12 = G[1][2] + G[2][1];
-  T Tn[3][3];  // Tn[k][i] = tension on the column-k edge, component i
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const T lw = cf.l(ph, k), mw = cf.m(ph, k);
-    Tn[k][k] = lw * tr + (mw + mw) * G[k][k];
-  }
-  {
-    Tn[0][1] = cf.m(ph, 0) * s01;
-    Tn[1][0] = cf.m(ph, 1) * s01;
-    Tn[0][2] = cf.m(ph, 0) * s02;
-    Tn[2][0] = cf.m(ph, 2) * s02;
-    Tn[1][2] = cf.m(ph, 1) * s12;
-    Tn[2][1] = cf.m(ph, 2) * s12;
-  }
-  if (EDGE) {
+  for (int k = 0; k < 3; ++k)
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
-      te->e0[p][i] += Tn[p][i];
-      te->em[p][q][i] += Tn[q][i];
-      te->el[r][i] += Tn[r][i];
+      const bool st = k == p ? (t & 1) == 0 : k == q ? true : first_r;
+      Te[E[k]][i] = st ? S[k][i] : Te[E[k]][i] + S[k][i];
     }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      F[0][i] -= Tn[p][i];
-      F[c1][i] += Tn[p][i] - Tn[q][i];
-      F[c2][i] += Tn[q][i] - Tn[r][i];
-      F[7][i] += Tn[r][i];
-    }
-  }
-  if (SIG) {
-    // |T| sigma_ik = h_k Tn[k][i]; |T| sigma : eps = sum_k hk[k] Tn[k] . Dr[k]
-    sg[0] += hk[0] * Tn[0][0];
-    sg[1] += hk[1] * Tn[1][1];
-    sg[2] += hk[2] * Tn[2][2];
-    sg[3] += hk[1] * Tn[1][2];
-    sg[4] += hk[0] * Tn[0][2];
-    sg[5] += hk[0] * Tn[0][1];
-    T e = T(0);
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      e += (UNIFORM ? T(1) : hk[k]) * (Tn[k][0] * Dr[k][0] + Tn[k][1] * Dr[k][1] + Tn[k][2] * Dr[k][2]);
-    en += e;
-  }
 }
 
-// Corner forces of a voxel from its edge tensions: each edge pulls its end corner and pushes
-// its start corner (corner index bits: x = 1, y = 2, z = 4).
+// The six tets of a voxel with codes `code`; lp, mp: phase moduli times the voxel scale
+template <typename T, int NPH>
+__device__ __forceinline__ void voxel_tets(const T (&D)[12][3], T (&Te)[12][3], unsigned code, const T (&lp)[NPH],
+                                           const T (&mp)[NPH]) {
+  const auto modulus = [&](int t, const T (&v)[NPH]) {
+    const unsigned cd = (code >> (2 * t)) & 3u;
+    T r = cd == 0u ? v[0] : T(0);
+    if (cd == 1u) r = v[1];
+    if (NPH > 2 && cd == 3u) r = v[NPH - 1];
+    return r;
+  };
+  voxel_tet<T, 0>(D, Te, modulus(0, lp), modulus(0, mp));
+  voxel_tet<T, 1>(D, Te, modulus(1, lp), modulus(1, mp));
+  voxel_tet<T, 2>(D, Te, modulus(2, lp), modulus(2, mp));
+  voxel_tet<T, 3>(D, Te, modulus(3, lp), modulus(3, mp));
+  voxel_tet<T, 4>(D, Te, modulus(4, lp), modulus(4, mp));
+  voxel_tet<T, 5>(D, Te, modulus(5, lp), modulus(5, mp));
+}
+
+// Stress sums of a voxel from its edge sums: int sigma_ik is component i summed over the edges
+// along k, up to the weight applied after the block sums.
 template <typename T>
-__device__ __forceinline__ void edge_forces(const EdgeT<T>& te, T (&F)[8][3]) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    F[0][i] = -(te.e0[0][i] + te.e0[1][i] + te.e0[2][i]);
-    F[7][i] = te.el[0][i] + te.el[1][i] + te.el[2][i];
-    F[1][i] = te.e0[0][i] - te.em[0][1][i] - te.em[0][2][i];
-    F[2][i] = te.e0[1][i] - te.em[1][0][i] - te.em[1][2][i];
-    F[4][i] = te.e0[2][i] - te.em[2][0][i] - te.em[2][1][i];
-    F[3][i] = te.em[0][1][i] + te.em[1][0][i] - te.el[2][i];
-    F[5][i] = te.em[0][2][i] + te.em[2][0][i] - te.el[1][i];
-    F[6][i] = te.em[1][2][i] + te.em[2][1][i] - te.el[0][i];
-  }
+__device__ __forceinline__ void voxel_stress_sums(const T (&Te)[12][3], T (&sg)[6]) {
+  const auto sum4 = [&](int k, int i) {
+    return (Te[4 * k][i] + Te[4 * k + 1][i]) + (Te[4 * k + 2][i] + Te[4 * k + 3][i]);
+  };
+  sg[0] += sum4(0, 0);
+  sg[1] += sum4(1, 1);
+  sg[2] += sum4(2, 2);
+  sg[3] += sum4(1, 2);
+  sg[4] += sum4(0, 2);
+  sg[5] += sum4(0, 1);
 }
 
-#ifndef XFFT_EDGE_FORCES
-#define XFFT_EDGE_FORCES 1  // corner forces from per-voxel edge tension sums
-#endif
+// Force component i on corner c (bits x = 1, y = 2, z = 4): an edge pulls its end corner and pushes
+// its start corner.
+template <bool UNIFORM, typename T>
+__device__ __forceinline__ T corner_force(const T (&Te)[12][3], const T (&wk)[3], int c, int i) {
+  const T ex = Te[cube_edge(c & 6, 0)][i], ey = Te[cube_edge(c & 5, 1)][i], ez = Te[cube_edge(c & 3, 2)][i];
+  T f;
+  if (UNIFORM) {
+    f = (c & 1) ? ex : -ex;
+    f = (c & 2) ? f + ey : f - ey;
+    f = (c & 4) ? f + ez : f - ez;
+  } else {
+    f = (c & 1) ? ex * wk[0] : ex * -wk[0];
+    f = f + ey * ((c & 2) ? wk[1] : -wk[1]);
+    f = f + ez * ((c & 4) ? wk[2] : -wk[2]);
+  }
+  return f;
+}
 
-template <typename T, bool TOTAL, bool SIG, bool UNIFORM, bool FUSED, int NPH>
+// Moduli factors of the edge form: uniform voxels use raw differences with |T| / h^2 in the moduli;
+// otherwise differences carry 1/h_k and corner forces the weights |T| / h_k.
+template <typename T, bool UNIFORM, int NPH>
+__device__ __forceinline__ void edge_moduli(const GridDev& g, const PhaseDev& ph, T (&l0)[NPH], T (&m0)[NPH]) {
+  const double w = UNIFORM ? g.vol_tet / (g.h[0] * g.h[0]) : 1.0;
+#pragma unroll
+  for (int p = 0; p < NPH; ++p) {
+    l0[p] = (T)(ph.lam[p] * w);
+    m0[p] = (T)(ph.mu[p] * w);
+  }
+}
+// eps_bar as it adds to the differences (raw differences carry a factor h)
+template <typename T, bool UNIFORM>
+__device__ __forceinline__ void edge_strain(const GridDev& g, const double* e, T (&Eb)[3][3]) {
+  const double rs = 0.70710678118654752440;
+  const double sc = UNIFORM ? g.h[0] : 1.0;
+  Eb[0][0] = (T)(e[0] * sc);
+  Eb[1][1] = (T)(e[1] * sc);
+  Eb[2][2] = (T)(e[2] * sc);
+  Eb[1][2] = Eb[2][1] = (T)(e[3] * rs * sc);
+  Eb[0][2] = Eb[2][0] = (T)(e[4] * rs * sc);
+  Eb[0][1] = Eb[1][0] = (T)(e[5] * rs * sc);
+}
+
+// The FP32 stencil.  A block of kTZ x kTY (16 x 16) threads owns one voxel column each (y, z), with a
+// halo row and column on the low side, and walks along x; node planes of d are staged in shared
+// memory one step ahead, forces on the plane's nodes are combined in shared memory and forces on
+// the next plane stay in registers, so every node force is written once with a plain store.
+//
+// What bounds it: instruction issue, then memory (78 bytes per voxel and right-hand side with the
+// fused update).  The voxel's twelve edges carry all its differences (those of the next plane are
+// kept: 24 subtractions per voxel) and its tension sums; cut tets take zero moduli by selects instead
+// of six branches with their own re-convergence; corner forces cross threads as 16-byte vectors
+// (three stores and three loads per voxel instead of twelve shuffles and twelve accesses).
+template <bool TOTAL, bool SIG, bool UNIFORM, bool FUSED, int NPH>
 __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
-    k_apply_uncut(const typename Store<T>::type* __restrict__ d, typename Store<T>::type* __restrict__ q,
-                  const ApplyArgs a, int nxchunks) {
-  typedef typename Store<T>::type S;
+    k_apply_uncut(const float* __restrict__ d, float* __restrict__ q, const ApplyArgs a, int nxchunks) {
   const int tz = threadIdx.x, ty = threadIdx.y;
   const int tid = tz + kTZ * ty;
   const int rhs = blockIdx.z / nxchunks;
@@ -293,16 +268,16 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
   const long long plane = (long long)n1 * n2;
   const int z0 = blockIdx.x * (kTZ - 1), y0 = blockIdx.y * (kTY - 1), x0 = xc * kCX;
   const int x1 = min(x0 + kCX, n0);
-  const S* dr = d + rhs * a.stride;
-  S* qr = q + rhs * a.stride;
+  const float* dr = d + rhs * a.stride;
+  float* qr = q + rhs * a.stride;
 
-  __shared__ Node4<T> P[2][kTY + 1][kTZ + 1];
-  __shared__ T Ys[2][3][kTY][kTZ];
-  __shared__ double red[7 * 32];
+  __shared__ float4 P[2][kTY + 1][kTZ + 1];  // node planes
+  __shared__ float4 C[3][kTY][kTZ];          // forces on the corners (dy, dz) = (0, 1), (1, 0), (1, 1)
 
   constexpr int kPlaneNodes = (kTY + 1) * (kTZ + 1);
   int ld_slot[2];
   long long ld_off[2];
+  bool slot_own[2];  // the block updates the plane nodes with 1 <= iy < kTY, 1 <= iz < kTZ
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     const int lin = tid + k * kTZ * kTY;
@@ -311,61 +286,33 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
     const int yy = ((y0 - 1 + iy) % n1 + n1) % n1;
     const int zz = ((z0 - 1 + iz) % n2 + n2) % n2;
     ld_off[k] = (long long)yy * n2 + zz;
+    slot_own[k] = FUSED && ld_slot[k] >= 0 && iy >= 1 && iy <= kTY - 1 && iz >= 1 && iz <= kTZ - 1 &&
+                  y0 - 1 + iy < n1 && z0 - 1 + iz < n2;
   }
   const int yg = y0 - 1 + ty, zg = z0 - 1 + tz;
   const int yv = (yg % n1 + n1) % n1, zv = (zg % n2 + n2) % n2;
   const bool own = ty >= 1 && tz >= 1 && yg < n1 && zg < n2;
 
-  T ih[3], hk[3];
+  float ih[3], wk[3], l0[NPH], m0[NPH], Eb[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    ih[k] = (T)(1.0 / g.h[k]);
-    hk[k] = (T)g.h[k];
+    ih[k] = (float)(1.0 / g.h[k]);
+    wk[k] = (float)(g.vol_tet / g.h[k]);
   }
-  // phase coefficients without the voxel scale (converted once; no FP64 work in the loop)
-  T lw0[NPH][3], mw0[NPH][3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const double wk = UNIFORM ? g.vol_tet / (g.h[0] * g.h[0]) : g.vol_tet / g.h[k];
-#pragma unroll
-    for (int ph = 0; ph < NPH; ++ph) {
-      lw0[ph][k] = (T)(a.ph.lam[ph] * wk);
-      mw0[ph][k] = (T)(a.ph.mu[ph] * wk);
-    }
-  }
-  T Eb[3][3] = {};
-  if (TOTAL) {
-    const double* e = a.eps + 6 * rhs;
-    const double rs = 0.70710678118654752440;
-    const double sc = UNIFORM ? g.h[0] : 1.0;  // raw differences carry a factor h
-    Eb[0][0] = (T)(e[0] * sc);
-    Eb[1][1] = (T)(e[1] * sc);
-    Eb[2][2] = (T)(e[2] * sc);
-    Eb[1][2] = Eb[2][1] = (T)(e[3] * rs * sc);
-    Eb[0][2] = Eb[2][0] = (T)(e[4] * rs * sc);
-    Eb[0][1] = Eb[1][0] = (T)(e[5] * rs * sc);
-  }
+  edge_moduli<float, UNIFORM, NPH>(g, a.ph, l0, m0);
+  if (TOTAL) edge_strain<float, UNIFORM>(g, a.eps + 6 * rhs, Eb);
 
-  // fused CG update: the block owns the plane nodes with 1 <= iy <= kTY-1, 1 <= iz <= kTZ-1
-  // inside the grid; it stores d_new and updates u there (other blocks only read them as halo)
-  const S* zr = FUSED ? static_cast<const S*>(a.fz) + rhs * a.stride : nullptr;
-  S* dnr = FUSED ? static_cast<S*>(a.fdnew) + rhs * a.stride : nullptr;
-  S* ur = FUSED ? static_cast<S*>(a.fu) + rhs * a.stride : nullptr;
-  const T fa = FUSED ? (T)a.st[rhs].alpha : T(0);
-  const T fb = FUSED ? (T)a.st[rhs].beta : T(0);
-  bool slot_own[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int lin = tid + k * kTZ * kTY;
-    const int iy = lin / (kTZ + 1), iz = lin - iy * (kTZ + 1);
-    slot_own[k] = ld_slot[k] >= 0 && iy >= 1 && iy <= kTY - 1 && iz >= 1 && iz <= kTZ - 1 &&
-                  y0 - 1 + iy < n1 && z0 - 1 + iz < n2;
-  }
+  // fused CG update: d_new = z + beta d_old, u += alpha d_old
+  const float* zr = FUSED ? static_cast<const float*>(a.fz) + rhs * a.stride : nullptr;
+  float* dnr = FUSED ? static_cast<float*>(a.fdnew) + rhs * a.stride : nullptr;
+  float* ur = FUSED ? static_cast<float*>(a.fu) + rhs * a.stride : nullptr;
+  const float fa = FUSED ? (float)a.st[rhs].alpha : 0.0f;
+  const float fb = FUSED ? (float)a.st[rhs].beta : 0.0f;
 
   // Two-stage plane pipeline: fetch() issues the global loads of a node plane into registers,
   // commit() (one step later, after the arithmetic of the current step was issued) forms the
   // fused update, stores the block's own nodes and fills the shared-memory plane.
-  T pf[2][9];  // per load slot: z (or d) 0..2, d_old 3..5, u 6..8
+  float pf[2][9];  // per load slot: z (or d) 0..2, d_old 3..5, u 6..8
   long long pf_nd[2] = {0, 0};
   bool pf_own[2] = {false, false};
   auto fetch = [&](int xp, bool own_plane) {
@@ -376,22 +323,22 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
         const long long nd = (long long)xp * plane + ld_off[k];
         pf_nd[k] = nd;
         if (FUSED) {
-          pf[k][0] = from_store<T>(zr[nd]);
-          pf[k][1] = from_store<T>(zr[N + nd]);
-          pf[k][2] = from_store<T>(zr[2 * N + nd]);
-          pf[k][3] = from_store<T>(dr[nd]);
-          pf[k][4] = from_store<T>(dr[N + nd]);
-          pf[k][5] = from_store<T>(dr[2 * N + nd]);
+          pf[k][0] = zr[nd];
+          pf[k][1] = zr[N + nd];
+          pf[k][2] = zr[2 * N + nd];
+          pf[k][3] = dr[nd];
+          pf[k][4] = dr[N + nd];
+          pf[k][5] = dr[2 * N + nd];
           pf_own[k] = own_plane && slot_own[k];
           if (pf_own[k]) {
-            pf[k][6] = from_store<T>(ur[nd]);
-            pf[k][7] = from_store<T>(ur[N + nd]);
-            pf[k][8] = from_store<T>(ur[2 * N + nd]);
+            pf[k][6] = ur[nd];
+            pf[k][7] = ur[N + nd];
+            pf[k][8] = ur[2 * N + nd];
           }
         } else {
-          pf[k][0] = from_store<T>(dr[nd]);
-          pf[k][1] = from_store<T>(dr[N + nd]);
-          pf[k][2] = from_store<T>(dr[2 * N + nd]);
+          pf[k][0] = dr[nd];
+          pf[k][1] = dr[N + nd];
+          pf[k][2] = dr[2 * N + nd];
         }
       }
     }
@@ -400,35 +347,55 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       if (ld_slot[k] >= 0) {
-        const int iy = ld_slot[k] / (kTZ + 1), iz = ld_slot[k] - iy * (kTZ + 1);
-        Node4<T> v;
+        float4 v;
         if (FUSED) {
           v.x = pf[k][0] + fb * pf[k][3];
           v.y = pf[k][1] + fb * pf[k][4];
           v.z = pf[k][2] + fb * pf[k][5];
           if (pf_own[k]) {
             const long long nd = pf_nd[k];
-            dnr[nd] = to_store(v.x);
-            dnr[N + nd] = to_store(v.y);
-            dnr[2 * N + nd] = to_store(v.z);
-            ur[nd] = to_store(pf[k][6] + fa * pf[k][3]);
-            ur[N + nd] = to_store(pf[k][7] + fa * pf[k][4]);
-            ur[2 * N + nd] = to_store(pf[k][8] + fa * pf[k][5]);
+            dnr[nd] = v.x;
+            dnr[N + nd] = v.y;
+            dnr[2 * N + nd] = v.z;
+            ur[nd] = pf[k][6] + fa * pf[k][3];
+            ur[N + nd] = pf[k][7] + fa * pf[k][4];
+            ur[2 * N + nd] = pf[k][8] + fa * pf[k][5];
           }
         } else {
           v.x = pf[k][0];
           v.y = pf[k][1];
           v.z = pf[k][2];
         }
-        v.w = T(0);
-        P[buf][iy][iz] = v;
+        v.w = 0.0f;
+        (&P[buf][0][0])[ld_slot[k]] = v;
       }
     }
   };
 
-  T pend[3] = {T(0), T(0), T(0)};
-  T en = T(0);
-  T sg[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+  float D[12][3];    // edge differences (times 1/h_k unless UNIFORM), plus eps_bar when TOTAL
+  float pend[4][3];  // corner forces on plane x + 1: [2 dy + dz][component]
+  float uo[4][3];    // plane x at the corners [2 dy + dz]
+  auto corners = [&](int buf, float (&u)[4][3]) {
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const float4 v = P[buf][ty + (c >> 1)][tz + (c & 1)];
+      u[c][0] = v.x;
+      u[c][1] = v.y;
+      u[c][2] = v.z;
+    }
+  };
+  auto diff = [&](int e, int k, const float (&hi)[3], const float (&lo)[3]) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      float v = hi[i] - lo[i];
+      if (!UNIFORM) v *= ih[k];
+      if (TOTAL) v += Eb[i][k];
+      D[e][i] = v;
+    }
+  };
+
+  float en = 0.0f;
+  float sg[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   const int xfirst = ((x0 - 1) % n0 + n0) % n0;
   fetch(xfirst, false);
   commit(0);
@@ -437,10 +404,20 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
   const long long yz = (long long)yv * n2 + zv;
   unsigned nx_code = a.code[(long long)xfirst * plane + yz];
   float nx_scale = a.scale ? a.scale[(long long)xfirst * plane + yz] : 1.0f;
+  __syncthreads();
+  corners(0, uo);
+  diff(cube_edge(0, 1), 1, uo[2], uo[0]);
+  diff(cube_edge(4, 1), 1, uo[3], uo[1]);
+  diff(cube_edge(0, 2), 2, uo[1], uo[0]);
+  diff(cube_edge(2, 2), 2, uo[3], uo[2]);
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int i = 0; i < 3; ++i) pend[c][i] = 0.0f;
   int xw = xfirst;  // the wrapped voxel index x0 - 1 + s, advanced without a division per step
   for (int s = 0; s <= x1 - x0; ++s, xw = xw + 1 >= n0 ? xw + 1 - n0 : xw + 1) {
     const unsigned code = nx_code;
-    const T sv = from_store<T>(nx_scale);
+    const float sv = nx_scale;
     commit((s + 1) & 1);  // plane x0 + s
     if (s + 1 <= x1 - x0) {
       const int x1w = xw + 1 >= n0 ? xw + 1 - n0 : xw + 1;  // voxel of the next step
@@ -450,97 +427,77 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
       if (a.scale) nx_scale = a.scale[(long long)x1w * plane + yz];
     }
     __syncthreads();
-    Node4<T> u[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) u[c] = P[(s + (c & 1)) & 1][ty + ((c >> 1) & 1)][tz + ((c >> 2) & 1)];
-    Coef<T, UNIFORM, NPH> cf;
-#pragma unroll
-    for (int ph = 0; ph < NPH; ++ph)
-#pragma unroll
-      for (int k = 0; k < (UNIFORM ? 1 : 3); ++k) {
-        cf.lw[ph][k] = lw0[ph][k] * sv;
-        cf.mw[ph][k] = mw0[ph][k] * sv;
-      }
-    T F[8][3];
-    T ven = T(0);
-    T vsg[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-#if XFFT_EDGE_FORCES
+    float un[4][3];
+    corners((s + 1) & 1, un);
+    diff(cube_edge(0, 0), 0, un[0], uo[0]);
+    diff(cube_edge(2, 0), 0, un[2], uo[2]);
+    diff(cube_edge(4, 0), 0, un[1], uo[1]);
+    diff(cube_edge(6, 0), 0, un[3], uo[3]);
+    diff(cube_edge(1, 1), 1, un[2], un[0]);
+    diff(cube_edge(5, 1), 1, un[3], un[1]);
+    diff(cube_edge(1, 2), 2, un[1], un[0]);
+    diff(cube_edge(3, 2), 2, un[3], un[2]);
+    float Te[12][3];
     {
-      EdgeT<T> te;
+      float lp[NPH], mp[NPH];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          te.e0[k][i] = te.el[k][i] = T(0);
-#pragma unroll
-          for (int l = 0; l < 3; ++l) te.em[k][l][i] = T(0);
-        }
-      tet_stencil<T, 0, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      tet_stencil<T, 1, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      tet_stencil<T, 2, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      tet_stencil<T, 3, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      tet_stencil<T, 4, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      tet_stencil<T, 5, TOTAL, SIG, UNIFORM, NPH, true>(u, F, code, cf, ih, hk, Eb, ven, vsg, &te);
-      edge_forces(te, F);
+      for (int ph = 0; ph < NPH; ++ph) {
+        lp[ph] = l0[ph] * sv;
+        mp[ph] = m0[ph] * sv;
+      }
+      voxel_tets<float, NPH>(D, Te, code, lp, mp);
     }
-#else
+    if (SIG && own && s >= 1) voxel_stress_sums(Te, sg);
+    float f0[3];  // force on the thread's own node (dy, dz) = (0, 0)
 #pragma unroll
-    for (int c = 0; c < 8; ++c) F[c][0] = F[c][1] = F[c][2] = T(0);
-    tet_stencil<T, 0, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-    tet_stencil<T, 1, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-    tet_stencil<T, 2, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-    tet_stencil<T, 3, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-    tet_stencil<T, 4, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-    tet_stencil<T, 5, TOTAL, SIG, UNIFORM, NPH>(u, F, code, cf, ih, hk, Eb, ven, vsg);
-#endif
-    if (SIG && own && s >= 1) {
-      en += ven;
-#pragma unroll
-      for (int k = 0; k < 6; ++k) sg[k] += vsg[k];
-    }
-    T G2[2][2][3];
-#pragma unroll
-    for (int dx = 0; dx < 2; ++dx)
-#pragma unroll
-      for (int dy = 0; dy < 2; ++dy)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const T up = shfl_up_t<T>(0xffffffffu, F[dx + 2 * dy + 4][i], 1, kTZ);
-          G2[dx][dy][i] = F[dx + 2 * dy][i] + up;
-        }
-#pragma unroll
-    for (int dx = 0; dx < 2; ++dx)
-#pragma unroll
-      for (int i = 0; i < 3; ++i) Ys[dx][i][ty][tz] = G2[dx][1][i];
-    __syncthreads();
-    if (own) {
-      T H0[3], H1[3];
+    for (int cc = 0; cc < 4; ++cc) {
+      const int c = (cc & 2) + 4 * (cc & 1);  // corner on plane x
+      float f[3];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        H0[i] = G2[0][0][i] + Ys[0][i][ty - 1][tz];
-        H1[i] = G2[1][0][i] + Ys[1][i][ty - 1][tz];
+        f[i] = pend[cc][i] + corner_force<UNIFORM>(Te, wk, c, i);
+        pend[cc][i] = corner_force<UNIFORM>(Te, wk, c + 1, i);
       }
-      if (s >= 1) {
-        const long long nd = (long long)xw * plane + (long long)yv * n2 + zv;
-        const T q0 = pend[0] + H0[0], q1 = pend[1] + H0[1], q2 = pend[2] + H0[2];
-        qr[nd] = to_store(q0);
-        qr[N + nd] = to_store(q1);
-        qr[2 * N + nd] = to_store(q2);
-        if (!SIG) en += q0 * u[0].x + q1 * u[0].y + q2 * u[0].z;  // <d, q> of this node
+      if (cc == 0) {
+        f0[0] = f[0];
+        f0[1] = f[1];
+        f0[2] = f[2];
+      } else {
+        C[cc - 1][ty][tz] = make_float4(f[0], f[1], f[2], 0.0f);
       }
+    }
+    __syncthreads();
+    if (own && s >= 1) {
+      const float4 fz = C[0][ty][tz - 1], fy = C[1][ty - 1][tz], fyz = C[2][ty - 1][tz - 1];
+      const long long nd = (long long)xw * plane + yz;
+      const float q0 = (f0[0] + fz.x) + (fy.x + fyz.x);
+      const float q1 = (f0[1] + fz.y) + (fy.y + fyz.y);
+      const float q2 = (f0[2] + fz.z) + (fy.z + fyz.z);
+      qr[nd] = q0;
+      qr[N + nd] = q1;
+      qr[2 * N + nd] = q2;
+      en += q0 * uo[0][0] + q1 * uo[0][1] + q2 * uo[0][2];  // <d, q> of this node
+    }
+    // plane x + 1 becomes plane x
 #pragma unroll
-      for (int i = 0; i < 3; ++i) pend[i] = H1[i];
+    for (int i = 0; i < 3; ++i) {
+      D[cube_edge(0, 1)][i] = D[cube_edge(1, 1)][i];
+      D[cube_edge(4, 1)][i] = D[cube_edge(5, 1)][i];
+      D[cube_edge(0, 2)][i] = D[cube_edge(1, 2)][i];
+      D[cube_edge(2, 2)][i] = D[cube_edge(3, 2)][i];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) uo[c][i] = un[c][i];
     }
   }
-  const double r2 = 1.41421356237309504880;
-  double v[7] = {to_double(en), to_double(sg[0]), to_double(sg[1]), to_double(sg[2]),
-                 to_double(sg[3]) * r2, to_double(sg[4]) * r2, to_double(sg[5]) * r2};
   double tot[7] = {};
   if (SIG) {
+    __shared__ double red[7 * 32];
+    const double ws = UNIFORM ? g.h[0] : g.vol_tet, r2 = 1.41421356237309504880;
+    const double v[7] = {(double)en, sg[0] * ws, sg[1] * ws, sg[2] * ws, sg[3] * ws * r2, sg[4] * ws * r2, sg[5] * ws * r2};
     block_sum<7>(v, red, tot);
   } else {
-    __shared__ T red1[kTZ * kTY];
-    tot[0] = block_sum1<T>(en, red1);
+    __shared__ float red1[kTZ * kTY];
+    tot[0] = block_sum1<float>(en, red1);
   }
   if (tid == 0) {
     const int bid = blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * xc);

@@ -34,38 +34,6 @@ struct TileShape {
 };
 TileShape pick_tile(const GridDev& g, int n_rhs);  // apply.cu
 
-// edge of the cube along axis k starting at corner c (bit k of c is 0): 4 k + the other two bits
-__host__ __device__ constexpr int cube_edge(int c, int k) {
-  return 4 * k + (k == 0 ? c >> 1 : k == 1 ? (c & 1) | ((c >> 2) << 1) : c & 3);
-}
-
-// One Kuhn tet: its tensions sigma e_k added to (or, as the edge's first contribution, stored in)
-// the edge sums Te.  l, m: lambda, mu of the tet (zero for a cut tet) times the voxel scale.
-template <typename T, int t>
-__device__ __forceinline__ void tile_tet(const T (&D)[12][3], T (&Te)[12][3], T l, T m) {
-  constexpr int p = perm_p(t), q = perm_q(t), r = perm_r(t);
-  constexpr int E[3] = {p == 0 ? cube_edge(0, 0) : q == 0 ? cube_edge(1 << p, 0) : cube_edge(6, 0),
-                        p == 1 ? cube_edge(0, 1) : q == 1 ? cube_edge(1 << p, 1) : cube_edge(5, 1),
-                        p == 2 ? cube_edge(0, 2) : q == 2 ? cube_edge(1 << p, 2) : cube_edge(3, 2)};
-  // the first tet that reaches a shared edge stores; p edges are shared by tets 2p and 2p + 1
-  constexpr bool first_r = t == 0 || t == 1 || t == 3;
-  const T tr = D[E[0]][0] + D[E[1]][1] + D[E[2]][2];
-  const T s01 = D[E[0]][1] + D[E[1]][0], s02 = D[E[0]][2] + D[E[2]][0], s12 = D[E[1]][2] + D[E[2]][1];
-  const T m2 = m + m;
-  const T lt = l * tr;
-  const T t01 = m * s01, t02 = m * s02, t12 = m * s12;
-  // sigma of the tet (times the common factor of l and m): column k is its tension on the edge
-  // along k, up to the weight w_k that the corner forces apply
-  const T S[3][3] = {{lt + m2 * D[E[0]][0], t01, t02}, {t01, lt + m2 * D[E[1]][1], t12}, {t02, t12, lt + m2 * D[E[2]][2]}};
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const bool st = k == p ? (t & 1) == 0 : k == q ? true : first_r;
-      Te[E[k]][i] = st ? S[k][i] : Te[E[k]][i] + S[k][i];
-    }
-}
-
 template <typename T, bool TOTAL, bool SIG, bool UNIFORM, bool FUSED, int NPH>
 __global__ void __launch_bounds__(kTileThreads, 3)
     k_apply_tile(const typename Store<T>::type* __restrict__ d, typename Store<T>::type* __restrict__ q,
@@ -89,30 +57,14 @@ __global__ void __launch_bounds__(kTileThreads, 3)
   __shared__ double red[7 * 32];
 
   const int iy = tid / tz, iz = tid - iy * tz;
-  T ih[3], wk[3], l0[NPH], m0[NPH];
+  T ih[3], wk[3], l0[NPH], m0[NPH], Eb[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     ih[k] = (T)(1.0 / g.h[k]);
     wk[k] = (T)(g.vol_tet / g.h[k]);
   }
-#pragma unroll
-  for (int ph = 0; ph < NPH; ++ph) {  // uniform voxels: raw differences, |T| / h^2 in the moduli
-    const double w = UNIFORM ? g.vol_tet / (g.h[0] * g.h[0]) : 1.0;
-    l0[ph] = (T)(a.ph.lam[ph] * w);
-    m0[ph] = (T)(a.ph.mu[ph] * w);
-  }
-  T Eb[3][3];
-  if (TOTAL) {
-    const double* e = a.eps + 6 * rhs;
-    const double rs = 0.70710678118654752440;
-    const double sc = UNIFORM ? g.h[0] : 1.0;  // raw differences carry a factor h
-    Eb[0][0] = (T)(e[0] * sc);
-    Eb[1][1] = (T)(e[1] * sc);
-    Eb[2][2] = (T)(e[2] * sc);
-    Eb[1][2] = Eb[2][1] = (T)(e[3] * rs * sc);
-    Eb[0][2] = Eb[2][0] = (T)(e[4] * rs * sc);
-    Eb[0][1] = Eb[1][0] = (T)(e[5] * rs * sc);
-  }
+  edge_moduli<T, UNIFORM, NPH>(g, a.ph, l0, m0);
+  if (TOTAL) edge_strain<T, UNIFORM>(g, a.eps + 6 * rhs, Eb);
   // fused CG update: d_new = z + beta d_old, u += alpha d_old at the nodes the item owns
   const S* zr = FUSED ? static_cast<const S*>(a.fz) + rhs * a.stride : nullptr;
   S* dnr = FUSED ? static_cast<S*>(a.fdnew) + rhs * a.stride : nullptr;
@@ -249,46 +201,13 @@ __global__ void __launch_bounds__(kTileThreads, 3)
           mp[ph] = a.scale ? m0[ph] * sv : m0[ph];
         }
         T Te[12][3];
-        auto modulus = [&](int t, const T (&v)[NPH]) {
-          const unsigned cd = (code >> (2 * t)) & 3u;
-          T r = cd == 0u ? v[0] : T(0);
-          if (cd == 1u) r = v[1];
-          if (NPH > 2 && cd == 3u) r = v[NPH - 1];
-          return r;
-        };
-        tile_tet<T, 0>(D, Te, modulus(0, lp), modulus(0, mp));
-        tile_tet<T, 1>(D, Te, modulus(1, lp), modulus(1, mp));
-        tile_tet<T, 2>(D, Te, modulus(2, lp), modulus(2, mp));
-        tile_tet<T, 3>(D, Te, modulus(3, lp), modulus(3, mp));
-        tile_tet<T, 4>(D, Te, modulus(4, lp), modulus(4, mp));
-        tile_tet<T, 5>(D, Te, modulus(5, lp), modulus(5, mp));
-        if (SIG) {  // int sigma_ik: the sum of component i over the edges along k, weighted at the end
-          auto sum4 = [&](int k, int i) {
-            return (Te[4 * k][i] + Te[4 * k + 1][i]) + (Te[4 * k + 2][i] + Te[4 * k + 3][i]);
-          };
-          sg[0] += sum4(0, 0);
-          sg[1] += sum4(1, 1);
-          sg[2] += sum4(2, 2);
-          sg[3] += sum4(1, 2);
-          sg[4] += sum4(0, 2);
-          sg[5] += sum4(0, 1);
-        }
-        // an edge pulls its end corner and pushes its start corner
+        voxel_tets<T, NPH>(D, Te, code, lp, mp);
+        if (SIG) voxel_stress_sums(Te, sg);
 #pragma unroll
         for (int c = 0; c < 8; ++c)
 #pragma unroll
           for (int i = 0; i < 3; ++i) {
-            const T ex = Te[cube_edge(c & 6, 0)][i], ey = Te[cube_edge(c & 5, 1)][i], ez = Te[cube_edge(c & 3, 2)][i];
-            T f;
-            if (UNIFORM) {
-              f = (c & 1) ? ex : -ex;
-              f = (c & 2) ? f + ey : f - ey;
-              f = (c & 4) ? f + ez : f - ez;
-            } else {
-              f = (c & 1) ? ex * wk[0] : ex * -wk[0];
-              f = f + ey * ((c & 2) ? wk[1] : -wk[1]);
-              f = f + ez * ((c & 4) ? wk[2] : -wk[2]);
-            }
+            const T f = corner_force<UNIFORM>(Te, wk, c, i);
             const int cc = (c & 2) + (c >> 2);  // 2 dy + dz
             if (c & 1) F1[cc][i] = f;
             else C[3 * cc + i][tid] = pend[cc][i] + f;
@@ -342,8 +261,8 @@ cudaError_t launch_uncut_nph(const typename Store<T>::type* d, typename Store<T>
     dim3 grid(gz, gy, gx * n_rhs);
 #define XFFT_LAUNCH(TOT, SG, FU)                                                             \
   do {                                                                                       \
-    if (uni) k_apply_uncut<T, TOT, SG, true, FU, NPH><<<grid, block, 0, s>>>(d, q, a, gx);    \
-    else k_apply_uncut<T, TOT, SG, false, FU, NPH><<<grid, block, 0, s>>>(d, q, a, gx);       \
+    if (uni) k_apply_uncut<TOT, SG, true, FU, NPH><<<grid, block, 0, s>>>(d, q, a, gx);    \
+    else k_apply_uncut<TOT, SG, false, FU, NPH><<<grid, block, 0, s>>>(d, q, a, gx);       \
   } while (0)
     if (a.fz) {
       if (sig) XFFT_LAUNCH(false, true, true);
