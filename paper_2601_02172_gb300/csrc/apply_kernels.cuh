@@ -264,8 +264,8 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
     atomicAdd(a.units_uncut, 1ULL);
   const GridDev& g = a.g;
   const int n0 = g.n0, n1 = g.n1, n2 = g.n2;
-  const long long N = g.N;
-  const long long plane = (long long)n1 * n2;
+  // element indices inside a right-hand side fit 32 bits (3 N <= 3 2^28)
+  const unsigned N = (unsigned)g.N, plane = (unsigned)(n1 * n2);
   const int z0 = blockIdx.x * (kTZ - 1), y0 = blockIdx.y * (kTY - 1), x0 = xc * kCX;
   const int x1 = min(x0 + kCX, n0);
   const float* dr = d + rhs * a.stride;
@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
 
   constexpr int kPlaneNodes = (kTY + 1) * (kTZ + 1);
   int ld_slot[2];
-  long long ld_off[2];
+  unsigned ld_off[2];
   bool slot_own[2];  // the block updates the plane nodes with 1 <= iy < kTY, 1 <= iz < kTZ
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
     const int iy = lin / (kTZ + 1), iz = lin - iy * (kTZ + 1);
     const int yy = ((y0 - 1 + iy) % n1 + n1) % n1;
     const int zz = ((z0 - 1 + iz) % n2 + n2) % n2;
-    ld_off[k] = (long long)yy * n2 + zz;
+    ld_off[k] = yy * n2 + zz;
     slot_own[k] = FUSED && ld_slot[k] >= 0 && iy >= 1 && iy <= kTY - 1 && iz >= 1 && iz <= kTZ - 1 &&
                   y0 - 1 + iy < n1 && z0 - 1 + iz < n2;
   }
@@ -313,14 +313,14 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
   // commit() (one step later, after the arithmetic of the current step was issued) forms the
   // fused update, stores the block's own nodes and fills the shared-memory plane.
   float pf[2][9];  // per load slot: z (or d) 0..2, d_old 3..5, u 6..8
-  long long pf_nd[2] = {0, 0};
+  unsigned pf_nd[2] = {0, 0};
   bool pf_own[2] = {false, false};
   auto fetch = [&](int xp, bool own_plane) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       pf_own[k] = false;
       if (ld_slot[k] >= 0) {
-        const long long nd = (long long)xp * plane + ld_off[k];
+        const unsigned nd = xp * plane + ld_off[k];
         pf_nd[k] = nd;
         if (FUSED) {
           pf[k][0] = zr[nd];
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
           v.y = pf[k][1] + fb * pf[k][4];
           v.z = pf[k][2] + fb * pf[k][5];
           if (pf_own[k]) {
-            const long long nd = pf_nd[k];
+            const unsigned nd = pf_nd[k];
             dnr[nd] = v.x;
             dnr[N + nd] = v.y;
             dnr[2 * N + nd] = v.z;
@@ -401,9 +401,9 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
   commit(0);
   fetch(xfirst + 1 == n0 ? 0 : xfirst + 1, x0 < x1);
   // the voxel's phase code and modulus scale are loaded one x step ahead as well
-  const long long yz = (long long)yv * n2 + zv;
-  unsigned nx_code = a.code[(long long)xfirst * plane + yz];
-  float nx_scale = a.scale ? a.scale[(long long)xfirst * plane + yz] : 1.0f;
+  const unsigned yz = yv * n2 + zv;
+  unsigned nx_code = a.code[xfirst * plane + yz];
+  float nx_scale = a.scale ? a.scale[xfirst * plane + yz] : 1.0f;
   __syncthreads();
   corners(0, uo);
   diff(cube_edge(0, 1), 1, uo[2], uo[0]);
@@ -423,8 +423,8 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
       const int x1w = xw + 1 >= n0 ? xw + 1 - n0 : xw + 1;  // voxel of the next step
       const int xn = xw + 2 >= n0 ? xw + 2 - n0 : xw + 2;  // plane x0 + s + 1
       fetch(xn, x0 + s + 1 < x1);
-      nx_code = a.code[(long long)x1w * plane + yz];
-      if (a.scale) nx_scale = a.scale[(long long)x1w * plane + yz];
+      nx_code = a.code[x1w * plane + yz];
+      if (a.scale) nx_scale = a.scale[x1w * plane + yz];
     }
     __syncthreads();
     float un[4][3];
@@ -445,7 +445,20 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
         lp[ph] = l0[ph] * sv;
         mp[ph] = m0[ph] * sv;
       }
-      voxel_tets<float, NPH>(D, Te, code, lp, mp);
+      // warps whose voxels each lie in one phase (most of them) need no selects
+      const bool one = code == 0u || code == 0x555u || (NPH > 2 && code == 0xfffu);
+      if (__all_sync(0xffffffffu, one)) {
+        const float l = code == 0u ? lp[0] : NPH > 2 && code == 0xfffu ? lp[NPH - 1] : lp[1];
+        const float m = code == 0u ? mp[0] : NPH > 2 && code == 0xfffu ? mp[NPH - 1] : mp[1];
+        voxel_tet<float, 0>(D, Te, l, m);
+        voxel_tet<float, 1>(D, Te, l, m);
+        voxel_tet<float, 2>(D, Te, l, m);
+        voxel_tet<float, 3>(D, Te, l, m);
+        voxel_tet<float, 4>(D, Te, l, m);
+        voxel_tet<float, 5>(D, Te, l, m);
+      } else {
+        voxel_tets<float, NPH>(D, Te, code, lp, mp);
+      }
     }
     if (SIG && own && s >= 1) voxel_stress_sums(Te, sg);
     float f0[3];  // force on the thread's own node (dy, dz) = (0, 0)
@@ -469,7 +482,7 @@ __global__ void __launch_bounds__(kTZ* kTY, XFFT_UNCUT_MINB)
     __syncthreads();
     if (own && s >= 1) {
       const float4 fz = C[0][ty][tz - 1], fy = C[1][ty - 1][tz], fyz = C[2][ty - 1][tz - 1];
-      const long long nd = (long long)xw * plane + yz;
+      const unsigned nd = xw * plane + yz;
       const float q0 = (f0[0] + fz.x) + (fy.x + fyz.x);
       const float q1 = (f0[1] + fz.y) + (fy.y + fyz.y);
       const float q2 = (f0[2] + fz.z) + (fy.z + fyz.z);
