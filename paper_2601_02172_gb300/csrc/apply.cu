@@ -287,11 +287,8 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
   const double* ur = u + rhs * a.stride;
   double E[6];
   mandel_to_tensor(a.eps + 6 * rhs, E);
-  double ih[3], w[3];
-  for (int k = 0; k < 3; ++k) {
-    ih[k] = 1.0 / g.h[k];
-    w[k] = g.vol_tet / g.h[k];
-  }
+  double ih[3];
+  for (int k = 0; k < 3; ++k) ih[k] = 1.0 / g.h[k];
   const double ivox = 1.0 / (6.0 * g.vol_tet);
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
        v += (long long)gridDim.x * blockDim.x) {
@@ -299,25 +296,34 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
     const int j = (int)((v / g.n2) % g.n1);
     const int i = (int)(v / ((long long)g.n1 * g.n2));
     double uu[8][3];
+#pragma unroll
     for (int c = 0; c < 8; ++c) {
       const long long nd = corner_node(g, i, j, k, c);
+#pragma unroll
       for (int x = 0; x < 3; ++x) uu[c][x] = ur[x * g.N + nd];
     }
     const double sv = a.scale ? (double)a.scale[v] : 1.0;
     double lms[kMaxPhases], mus[kMaxPhases];
+#pragma unroll
     for (int p = 0; p < kMaxPhases; ++p) {
       lms[p] = a.ph.lam[p] * sv;
       mus[p] = a.ph.mu[p] * sv;
     }
-    double F[8][3] = {};
-    double en = 0.0, sg[6] = {0, 0, 0, 0, 0, 0};
-    const unsigned code = a.code[v];
-    tet_uncut<double, 0, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
-    tet_uncut<double, 1, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
-    tet_uncut<double, 2, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
-    tet_uncut<double, 3, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
-    tet_uncut<double, 4, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
-    tet_uncut<double, 5, true>(uu, F, code, lms, mus, ih, w, g.vol_tet, E, en, sg);
+    // the voxel's edge differences (with eps_bar) and tension sums, as in the stencil
+    double D[12][3], Te[12][3], sg[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (!(c & (1 << ax))) {
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+            D[cube_edge(c, ax)][x] = (uu[c | (1 << ax)][x] - uu[c][x]) * ih[ax] + sym_at(E, x, ax);
+        }
+    voxel_tets<double, kMaxPhases>(D, Te, a.code[v], lms, mus);
+    voxel_stress_sums(Te, sg);
+#pragma unroll
+    for (int x = 0; x < 6; ++x) sg[x] *= g.vol_tet;
     const double r2 = 1.41421356237309504880;
     double* o = out + (long long)rhs * 6 * g.N;
     o[0 * g.N + v] = sg[0] * ivox;

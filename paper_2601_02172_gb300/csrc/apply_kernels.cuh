@@ -28,21 +28,6 @@ constexpr int kCX = XFFT_UNCUT_CX;  // output planes per block along x
 #define XFFT_UNCUT_MINB 2  // resident blocks per SM asked of the FP32 uncut kernel
 #endif
 
-template <typename T>
-__device__ __forceinline__ T cut_real(const CutData& cd, int f, int e);
-template <>
-__device__ __forceinline__ double cut_real<double>(const CutData& cd, int f, int e) {
-  return cd.dp[(long long)f * cd.ncut + e];
-}
-template <>
-__device__ __forceinline__ float cut_real<float>(const CutData& cd, int f, int e) {
-  return cd.fp[(long long)f * cd.ncut + e];
-}
-template <>
-__device__ __forceinline__ dw cut_real<dw>(const CutData& cd, int f, int e) {
-  return dw(cd.dp[(long long)f * cd.ncut + e]);
-}
-
 // symmetric tensor stored as (00, 11, 22, 12, 02, 01)
 template <typename T>
 __device__ __forceinline__ T sym_at(const T (&s)[6], int i, int j) {
@@ -77,58 +62,6 @@ __device__ __forceinline__ void iso_stress(const T (&e)[6], T lam, T mu, T (&s)[
 template <typename T>
 __device__ __forceinline__ T ddot(const T (&s)[6], const T (&e)[6]) {
   return s[0] * e[0] + s[1] * e[1] + s[2] * e[2] + T(2) * (s[3] * e[3] + s[4] * e[4] + s[5] * e[5]);
-}
-
-// One uncut Kuhn tet t of a voxel with corner displacements u: adds its corner forces to F and
-// its energy/stress integrals to the accumulators.
-template <typename T, int t, bool TOTAL>
-__device__ __forceinline__ void tet_uncut(const T (&u)[8][3], T (&F)[8][3], unsigned code,
-                                          const T (&lm)[kMaxPhases], const T (&mu2)[kMaxPhases],
-                                          const T (&ih)[3],
-                                          const T (&w)[3], T vol, const T (&E)[6], T& en,
-                                          T (&sg)[6]) {
-  constexpr int p = perm_p(t), q = perm_q(t), r = perm_r(t);
-  constexpr int c1 = tet_c1(t), c2 = tet_c2(t);
-  const unsigned cd = (code >> (2 * t)) & 3u;
-  if (cd == kCodeCut) return;
-  const T lam = lm[code_phase(cd)], mu = mu2[code_phase(cd)];
-  T H[3][3];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    H[i][p] = (u[c1][i] - u[0][i]) * ih[p];
-    H[i][q] = (u[c2][i] - u[c1][i]) * ih[q];
-    H[i][r] = (u[7][i] - u[c2][i]) * ih[r];
-  }
-  T e[6];
-  e[0] = H[0][0];
-  e[1] = H[1][1];
-  e[2] = H[2][2];
-  e[3] = T(0.5) * (H[1][2] + H[2][1]);
-  e[4] = T(0.5) * (H[0][2] + H[2][0]);
-  e[5] = T(0.5) * (H[0][1] + H[1][0]);
-  if (TOTAL) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) e[k] += E[k];
-  }
-  T s[6];
-  iso_stress(e, lam, mu, s);
-  en += vol * ddot(s, e);
-  sg[0] += vol * s[0];
-  sg[1] += vol * s[1];
-  sg[2] += vol * s[2];
-  sg[3] += vol * s[3];
-  sg[4] += vol * s[4];
-  sg[5] += vol * s[5];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const T tp = w[p] * sym_at(s, i, p);
-    const T tq = w[q] * sym_at(s, i, q);
-    const T tr = w[r] * sym_at(s, i, r);
-    F[0][i] -= tp;
-    F[c1][i] += tp - tq;
-    F[c2][i] += tq - tr;
-    F[7][i] += tr;
-  }
 }
 
 // ---------------------------------------------------------------- uncut stencil

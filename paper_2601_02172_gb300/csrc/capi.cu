@@ -91,7 +91,6 @@ struct xfft_ctx {
   int nX = -1, ncut = -1;
   int* cut_ip = nullptr;
   double* cut_dp = nullptr;
-  float* cut_fp = nullptr;
   int4* cut_n4 = nullptr;
   int4* cut_e4 = nullptr;
   double* cut_r64 = nullptr;
@@ -247,7 +246,6 @@ static CutData cutdata(const xfft_ctx* c) {
   CutData cd;
   cd.ip = c->cut_ip;
   cd.dp = c->cut_dp;
-  cd.fp = c->cut_fp;
   cd.ncut = c->ncut;
   cd.n4 = c->cut_n4;
   cd.e4 = c->cut_e4;
@@ -398,7 +396,6 @@ static void free_micro(xfft_ctx* c) {
   dfree(c, c->scale);
   dfree(c, c->cut_ip);
   dfree(c, c->cut_dp);
-  dfree(c, c->cut_fp);
   dfree(c, c->cut_n4);
   dfree(c, c->cut_e4);
   dfree(c, c->cut_r64);
@@ -571,7 +568,6 @@ extern "C" xfft_status xfft_set_microstructure_phases(xfft_ctx* c, int n_levelse
   CU(dalloc(c, &c->enr_nodes, c->nX));
   CU(dalloc(c, &c->cut_ip, (size_t)kCutInts * c->ncut));
   CU(dalloc(c, &c->cut_dp, (size_t)kCutReals * c->ncut));
-  CU(dalloc(c, &c->cut_fp, (size_t)kCutReals * c->ncut));
   {
     int* chunk_tmp = nullptr;
     CU(dalloc(c, &chunk_tmp, 2 * (size_t)chunk_ints(c->ncut)));
@@ -605,7 +601,6 @@ extern "C" xfft_status xfft_set_microstructure_phases(xfft_ctx* c, int n_levelse
     CU(cudaStreamSynchronize(s));
     if (hbad) return fail(XFFT_EBREAKDOWN, "an enriched 3x3 block is not positive definite");
   }
-  CU(launch_cut_to_float(c->cut_dp, c->cut_fp, (long long)kCutReals * c->ncut, s));
   CU(dalloc(c, &c->cut_n4, c->ncut));
   CU(dalloc(c, &c->cut_e4, c->ncut));
   CU(dalloc(c, &c->cut_r64, (size_t)kRec * c->ncut));

@@ -43,117 +43,94 @@ struct Moments {
   double M[10];
 };
 
-XFFT_HD inline double det4(const double b[4][4]) {
-  // Laplace expansion along the first row
-  double d = 0.0;
-#pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    int cols[3];
-    int q = 0;
-#pragma unroll
-    for (int cc = 0; cc < 4; ++cc)
-      if (cc != c) cols[q++] = cc;
-    const double m3 = b[1][cols[0]] * (b[2][cols[1]] * b[3][cols[2]] - b[2][cols[2]] * b[3][cols[1]])
-                    - b[1][cols[1]] * (b[2][cols[0]] * b[3][cols[2]] - b[2][cols[2]] * b[3][cols[0]])
-                    + b[1][cols[2]] * (b[2][cols[0]] * b[3][cols[1]] - b[2][cols[1]] * b[3][cols[0]]);
-    d += ((c & 1) ? -1.0 : 1.0) * b[0][c] * m3;
-  }
-  return d;
+// Add the moments of a sub-tetrahedron of volume v: int N_b = v/4 S_b and int N_b N_c =
+// v/20 (pp_bc + S_b S_c), where S_b = sum_v beta_vb and pp_bc = sum_v beta_vb beta_vc over its
+// vertices' parent barycentric coordinates beta_v.  Arguments: S, then the packed pp.
+XFFT_HD inline void add_subtet(Moments& acc, double v, double s0, double s1, double s2, double s3, double p00,
+                               double p01, double p02, double p03, double p11, double p12, double p13, double p22,
+                               double p23, double p33) {
+  const double v4 = 0.25 * v, v20 = 0.05 * v;
+  acc.m[0] += v4 * s0;
+  acc.m[1] += v4 * s1;
+  acc.m[2] += v4 * s2;
+  acc.m[3] += v4 * s3;
+  acc.M[0] += v20 * (p00 + s0 * s0);
+  acc.M[1] += v20 * (p01 + s0 * s1);
+  acc.M[2] += v20 * (p02 + s0 * s2);
+  acc.M[3] += v20 * (p03 + s0 * s3);
+  acc.M[4] += v20 * (p11 + s1 * s1);
+  acc.M[5] += v20 * (p12 + s1 * s2);
+  acc.M[6] += v20 * (p13 + s1 * s3);
+  acc.M[7] += v20 * (p22 + s2 * s2);
+  acc.M[8] += v20 * (p23 + s2 * s3);
+  acc.M[9] += v20 * (p33 + s3 * s3);
 }
 
-// Add the moments of the sub-tetrahedron whose vertices have parent barycentric coordinates
-// beta[v][.]: its volume is |det beta| |T|, int N_b = vol/4 sum_v beta_vb and
-// int N_b N_c = vol/20 (sum_v beta_vb beta_vc + (sum_v beta_vb)(sum_v beta_vc)).
-XFFT_HD inline void add_subtet(Moments& acc, const double b0[4], const double b1[4],
-                                  const double b2[4], const double b3[4], double vol) {
-  const double B[4][4] = {{b0[0], b0[1], b0[2], b0[3]},
-                          {b1[0], b1[1], b1[2], b1[3]},
-                          {b2[0], b2[1], b2[2], b2[3]},
-                          {b3[0], b3[1], b3[2], b3[3]}};
-  const double vs = fabs(det4(B)) * vol;
-  double S[4];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) S[c] = B[0][c] + B[1][c] + B[2][c] + B[3][c];
-#pragma unroll
-  for (int c = 0; c < 4; ++c) acc.m[c] += 0.25 * vs * S[c];
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int c = b; c < 4; ++c) {
-      const double pp = B[0][b] * B[0][c] + B[1][b] * B[1][c] + B[2][b] * B[2][c] + B[3][b] * B[3][c];
-      acc.M[midx(b, c)] += vs / 20.0 * (pp + S[b] * S[c]);
-    }
-}
+XFFT_HD inline double pick4(const double L[4], int i) { return i < 2 ? (i ? L[1] : L[0]) : (i == 3 ? L[3] : L[2]); }
 
-XFFT_HD inline void unit_bary(int a, double out[4]) {
-#pragma unroll
-  for (int c = 0; c < 4; ++c) out[c] = (c == a) ? 1.0 : 0.0;
-}
-
-// barycentric point where L_h = 0 on the edge (a, b) (L_a L_b < 0), or vertex a if L_a = 0
-XFFT_HD inline void edge_point(const double L[4], int a, int b, double out[4]) {
-  if (L[a] == 0.0) {
-    unit_bary(a, out);
-    return;
-  }
-  const double t = L[a] / (L[a] - L[b]);
-#pragma unroll
-  for (int c = 0; c < 4; ++c) out[c] = 0.0;
-  out[a] = 1.0 - t;
-  out[b] = t;
-}
-
-// Moments of side s (+1: s L_h >= 0) of a cut tet with nodal values L.
-//   one strictly positive vertex a:   tet (a, edge points to the others)
-//   one strictly negative vertex q:   prism (other three) -> (their edge points to q)
-//   two and two:                       prism (a1, x11, x12) -> (a2, x21, x22)
-XFFT_HD inline void side_moments(const double L[4], int s, double vol, Moments& out) {
-#pragma unroll
+// Moments of side s (+1: s L_h >= 0) of a cut tet with nodal values L, its vertices in the order
+// perm (vertex perm[k] of the tet is vertex k here), which brings every cut to one of three forms:
+//   one strictly positive vertex (first):  tet of it and the edge points to the others
+//   one strictly negative vertex (first):  prism (other three) -> (their edge points to it)
+//   two and two (positive ones first):     prism (a1, x11, x12) -> (a2, x21, x22)
+// An edge point is (1 - t) v + t w with L = 0 there (a vertex with L = 0 is its own edge point).  The
+// prisms split into the three tets of consecutive points; the volumes |det beta| are products of the
+// edge coordinates.  Nothing is indexed by data, so on the GPU all of it stays in registers.
+XFFT_HD inline void side_moments_ordered(const double L[4], int s, double vol, Moments& out, int perm[4]) {
   for (int c = 0; c < 4; ++c) out.m[c] = 0.0;
-#pragma unroll
   for (int c = 0; c < 10; ++c) out.M[c] = 0.0;
-  int P[4], Q[4], Z[4];
-  int np = 0, nq = 0, nz = 0;
-  for (int a = 0; a < 4; ++a) {
-    const double x = s * L[a];
-    if (x > 0.0)
-      P[np++] = a;
-    else if (x < 0.0)
-      Q[nq++] = a;
-    else
-      Z[nz++] = a;
-  }
-  double v[6][4];
-  if (np == 1) {
-    const int a = P[0];
-    unit_bary(a, v[0]);
-    int k = 1;
-    for (int i = 0; i < nq; ++i) edge_point(L, a, Q[i], v[k++]);
-    for (int i = 0; i < nz; ++i) unit_bary(Z[i], v[k++]);
-    add_subtet(out, v[0], v[1], v[2], v[3], vol);
-  } else if (nq == 1) {
-    const int q = Q[0];
-    int k = 0;
-    for (int a = 0; a < 4; ++a) {
-      if (a == q) continue;
-      unit_bary(a, v[k]);
-      edge_point(L, a, q, v[3 + k]);
-      ++k;
+  const double x0 = s * L[0], x1 = s * L[1], x2 = s * L[2], x3 = s * L[3];
+  const int np = (x0 > 0.0) + (x1 > 0.0) + (x2 > 0.0) + (x3 > 0.0);
+  const int nq = (x0 < 0.0) + (x1 < 0.0) + (x2 < 0.0) + (x3 < 0.0);
+  if (np == 1 || nq == 1) {
+    const double g = np == 1 ? 1.0 : -1.0;  // the lone vertex is the one with g x > 0
+    const int a = g * x0 > 0.0 ? 0 : g * x1 > 0.0 ? 1 : g * x2 > 0.0 ? 2 : 3;
+    perm[0] = a;
+    perm[1] = a == 0 ? 1 : 0;
+    perm[2] = a <= 1 ? 2 : 1;
+    perm[3] = a <= 2 ? 3 : 2;
+    const double la = pick4(L, a), l0 = pick4(L, perm[1]), l1 = pick4(L, perm[2]), l2 = pick4(L, perm[3]);
+    if (np == 1) {
+      const double t0 = la / (la - l0), t1 = la / (la - l1), t2 = la / (la - l2);
+      const double u0 = 1.0 - t0, u1 = 1.0 - t1, u2 = 1.0 - t2;
+      add_subtet(out, t0 * t1 * t2 * vol, 1.0 + u0 + u1 + u2, t0, t1, t2, 1.0 + u0 * u0 + u1 * u1 + u2 * u2, u0 * t0,
+                 u1 * t1, u2 * t2, t0 * t0, 0.0, 0.0, t1 * t1, 0.0, t2 * t2);
+    } else {
+      const double t0 = l0 / (l0 - la), t1 = l1 / (l1 - la), t2 = l2 / (l2 - la);
+      const double u0 = 1.0 - t0, u1 = 1.0 - t1, u2 = 1.0 - t2;
+      const double c0 = u0 * t0, c1 = u1 * t1, c2 = u2 * t2;
+      add_subtet(out, t0 * vol, t0, 1.0 + u0, 1.0, 1.0, t0 * t0, c0, 0.0, 0.0, 1.0 + u0 * u0, 0.0, 0.0, 1.0, 0.0, 1.0);
+      add_subtet(out, u0 * t1 * vol, t0 + t1, u0, 1.0 + u1, 1.0, t0 * t0 + t1 * t1, c0, c1, 0.0, u0 * u0, 0.0, 0.0,
+                 1.0 + u1 * u1, 0.0, 1.0);
+      add_subtet(out, u0 * u1 * t2 * vol, t0 + t1 + t2, u0, u1, 1.0 + u2, t0 * t0 + t1 * t1 + t2 * t2, c0, c1, c2,
+                 u0 * u0, 0.0, 0.0, u1 * u1, 0.0, 1.0 + u2 * u2);
     }
-    add_subtet(out, v[0], v[1], v[2], v[3], vol);
-    add_subtet(out, v[1], v[2], v[3], v[4], vol);
-    add_subtet(out, v[2], v[3], v[4], v[5], vol);
   } else {
-    const int a1 = P[0], a2 = P[1], b1 = Q[0], b2 = Q[1];
-    unit_bary(a1, v[0]);
-    edge_point(L, a1, b1, v[1]);
-    edge_point(L, a1, b2, v[2]);
-    unit_bary(a2, v[3]);
-    edge_point(L, a2, b1, v[4]);
-    edge_point(L, a2, b2, v[5]);
-    add_subtet(out, v[0], v[1], v[2], v[3], vol);
-    add_subtet(out, v[1], v[2], v[3], v[4], vol);
-    add_subtet(out, v[2], v[3], v[4], v[5], vol);
+    perm[0] = x0 > 0.0 ? 0 : x1 > 0.0 ? 1 : 2;
+    perm[1] = x3 > 0.0 ? 3 : x2 > 0.0 ? 2 : 1;
+    perm[2] = x0 < 0.0 ? 0 : x1 < 0.0 ? 1 : 2;
+    perm[3] = x3 < 0.0 ? 3 : x2 < 0.0 ? 2 : 1;
+    const double a1 = pick4(L, perm[0]), a2 = pick4(L, perm[1]), b1 = pick4(L, perm[2]), b2 = pick4(L, perm[3]);
+    const double t11 = a1 / (a1 - b1), t12 = a1 / (a1 - b2), t21 = a2 / (a2 - b1), t22 = a2 / (a2 - b2);
+    const double u11 = 1.0 - t11, u12 = 1.0 - t12, u21 = 1.0 - t21, u22 = 1.0 - t22;
+    const double c11 = u11 * t11, c12 = u12 * t12, c21 = u21 * t21, c22 = u22 * t22;
+    add_subtet(out, t11 * t12 * vol, 1.0 + u11 + u12, 1.0, t11, t12, 1.0 + u11 * u11 + u12 * u12, 0.0, c11, c12, 1.0,
+               0.0, 0.0, t11 * t11, 0.0, t12 * t12);
+    add_subtet(out, u11 * t12 * t21 * vol, u11 + u12, 1.0 + u21, t11 + t21, t12, u11 * u11 + u12 * u12, 0.0, c11, c12,
+               1.0 + u21 * u21, c21, 0.0, t11 * t11 + t21 * t21, 0.0, t12 * t12);
+    add_subtet(out, u12 * t21 * t22 * vol, u12, 1.0 + u21 + u22, t21, t12 + t22, u12 * u12, 0.0, 0.0, c12,
+               1.0 + u21 * u21 + u22 * u22, c21, c22, t21 * t21, 0.0, t12 * t12 + t22 * t22);
+  }
+}
+
+// the same in the tet's own vertex order
+XFFT_HD inline void side_moments(const double L[4], int s, double vol, Moments& out) {
+  Moments o;
+  int perm[4];
+  side_moments_ordered(L, s, vol, o, perm);
+  for (int b = 0; b < 4; ++b) {
+    out.m[perm[b]] = o.m[b];
+    for (int c = b; c < 4; ++c) out.M[midx(perm[b], perm[c])] = o.M[midx(b, c)];
   }
 }
 
@@ -250,22 +227,29 @@ XFFT_HD inline void cut_scaling_terms(const double L[4], const double gr[4][3], 
       c[b] = fabs(L[b]) - s * L[b];
       for (int x = 0; x < 3; ++x) gam[x] += c[b] * gr[b][x];
     }
+    // sum_bc M_bc V_ab[x] V_ac[y] = Q g_x g_y + R_a (g_x gamma_y + gamma_x g_y) + M_aa gamma_x gamma_y with
+    // R_a = sum_c M_ac c_c and Q = sum_b c_b R_b: a tenth of the operations of the double sum
     const double* M = Mp[si];
+    double R[4], Q = 0.0;
     for (int a = 0; a < 4; ++a) {
-      double V[4][3];
-      for (int b = 0; b < 4; ++b)
-        for (int x = 0; x < 3; ++x) V[b][x] = c[b] * gr[a][x] + (a == b ? gam[x] : 0.0);
-      for (int b = 0; b < 4; ++b)
-        for (int cc = 0; cc < 4; ++cc) {
-          const double w = M[midx(b, cc)];
-          const double dot = V[b][0] * V[cc][0] + V[b][1] * V[cc][1] + V[b][2] * V[cc][2];
-          for (int x = 0; x < 3; ++x) acc[a][x] += 0.5 * w * (dot + V[b][x] * V[cc][x]);
-          if (want_off) {
-            off[a][0] += 0.5 * w * V[b][0] * V[cc][1];
-            off[a][1] += 0.5 * w * V[b][0] * V[cc][2];
-            off[a][2] += 0.5 * w * V[b][1] * V[cc][2];
-          }
-        }
+      R[a] = M[midx(a, 0)] * c[0] + M[midx(a, 1)] * c[1] + M[midx(a, 2)] * c[2] + M[midx(a, 3)] * c[3];
+      Q += c[a] * R[a];
+    }
+    for (int a = 0; a < 4; ++a) {
+      double h[3], k[3];  // Q g + R_a gamma and R_a g + M_aa gamma
+      for (int x = 0; x < 3; ++x) {
+        h[x] = Q * gr[a][x] + R[a] * gam[x];
+        k[x] = R[a] * gr[a][x] + M[midx(a, a)] * gam[x];
+      }
+      double T[3];
+      for (int x = 0; x < 3; ++x) T[x] = gr[a][x] * h[x] + gam[x] * k[x];
+      const double tr = T[0] + T[1] + T[2];
+      for (int x = 0; x < 3; ++x) acc[a][x] += 0.5 * (tr + T[x]);
+      if (want_off) {
+        off[a][0] += 0.5 * (gr[a][0] * h[1] + gam[0] * k[1]);
+        off[a][1] += 0.5 * (gr[a][0] * h[2] + gam[0] * k[2]);
+        off[a][2] += 0.5 * (gr[a][1] * h[2] + gam[1] * k[2]);
+      }
     }
   }
 }

@@ -78,6 +78,29 @@ struct Store<dw> {
   typedef double type;
 };
 
+// x = hi + lo with hi = x rounded to a float and lo the remainder rounded to a float, by integer
+// operations on the bits of x: the FP64 unit, which conversions and the subtraction would occupy (four
+// instructions of 16 clocks each), was most of the double-word cut kernel's time (92 loads per tet and
+// right-hand side).  hi: the low 29 mantissa bits rounded off, exponent rebiased; lo: those bits as a
+// signed integer times 2^(e - 1075).  Outside 2^-73 .. 2^126 (and for Inf and NaN) the FP64 way.
+__device__ __forceinline__ dw dw_split(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+  dw r;
+  if (e - 950u < 200u) {
+    const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+    const unsigned h = (unsigned)((b + 0x10000000ULL) >> 29) - (896u << 23);
+    const int l = ((int)((unsigned)b << 3)) >> 3;
+    r.hi = __uint_as_float((h & 0x7fffffffu) | sign);
+    r.lo = __int2float_rn(l) * __uint_as_float(((e - 948u) << 23) | sign);
+  } else if ((b << 1) == 0) {
+    r.hi = r.lo = 0.0f;
+  } else {
+    r = dw(x);
+  }
+  return r;
+}
+
 // storage -> compute and compute -> storage conversions
 template <typename T, typename S>
 __device__ __forceinline__ T from_store(S x) {
@@ -85,7 +108,7 @@ __device__ __forceinline__ T from_store(S x) {
 }
 template <>
 __device__ __forceinline__ dw from_store<dw, double>(double x) {
-  return dw(x);
+  return dw_split(x);
 }
 template <>
 __device__ __forceinline__ dw from_store<dw, float>(float x) {

@@ -394,15 +394,23 @@ __global__ void k_cut_geometry(const double* __restrict__ Ls, int nL, int* __res
     classify_tet(pv, nL, &pm, &pp, &two);
     ip[kCutFieldPhases * ncut + e] = pm | (pp << 8);
     double L[4];
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
-      L[a] = tv[pm][a];
+      L[a] = pm == 0 ? tv[0][a] : tv[kMaxPhases - 2][a];
       dp[cut_f_L(a) * (long long)ncut + e] = L[a];
     }
+    // the moments come in the cut's own vertex order; their fields are addressed through it
+#pragma unroll
     for (int si = 0; si < 2; ++si) {
       Moments mo;
-      side_moments(L, si == 0 ? +1 : -1, g.vol_tet, mo);
-      for (int b = 0; b < 4; ++b) dp[cut_f_m(si, b) * (long long)ncut + e] = mo.m[b];
-      for (int c = 0; c < 10; ++c) dp[cut_f_M(si, c) * (long long)ncut + e] = mo.M[c];
+      int perm[4];
+      side_moments_ordered(L, si == 0 ? +1 : -1, g.vol_tet, mo, perm);
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        dp[cut_f_m(si, perm[b]) * (long long)ncut + e] = mo.m[b];
+#pragma unroll
+        for (int c = b; c < 4; ++c) dp[cut_f_M(si, midx(perm[b], perm[c])) * (long long)ncut + e] = mo.M[midx(b, c)];
+      }
     }
   }
 }
@@ -488,8 +496,11 @@ __global__ void k_cut_matrix(const int* __restrict__ ip, const double* __restric
   }
 }
 
-// Reduced element records (apply_cut_el.cuh): with D0^-1/2 = dsc folded in, l_b and p_b / 2 from
-// v_sb = (m.c)_s g_b + m_sb gamma_s, the enriched block from the cached-matrix entries.
+// Reduced element records (apply_cut_el.cuh), formed in FP64: with D0^-1/2 = dsc folded in, l_b and
+// p_b / 2 from v_sb = (m.c)_s g_b + m_sb gamma_s, and per side the enriched block of the vertices a, b
+//   K_xy = lambda A_xy + mu (A_yx + delta_xy tr A),
+//   A = g_a (x) (Q g_b + R_b gamma) + gamma (x) (R_a g_b + M_ab gamma)
+// (SideW's weights; about 1100 FP64 operations per tet, against 5000 entry by entry).
 __global__ void __launch_bounds__(128) k_cut_elements(const int* __restrict__ ip, const double* __restrict__ dp,
                                                       const double* __restrict__ isD, int nX, int ncut, GridDev g,
                                                       PhaseDev ph, const float* __restrict__ scale,
@@ -502,23 +513,29 @@ __global__ void __launch_bounds__(128) k_cut_elements(const int* __restrict__ ip
     double gr[4][3];
     tet_grads<double>(t, ih, gr);
     double L[4], dsc[4][3];
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
       L[a] = dp[(long long)cut_f_L(a) * ncut + e];
       const int j = ip[(4 + a) * ncut + e];
+#pragma unroll
       for (int x = 0; x < 3; ++x) dsc[a][x] = isD[(long long)x * nX + j];
     }
     const double sv = scale ? (double)scale[vox] : 1.0;
     SideW w[2];
     double lam = 0.0, mu = 0.0, l[4][3] = {}, p[4][3] = {};
+#pragma unroll
     for (int si = 0; si < 2; ++si) {
       const int f = si == 0 ? cut_phase_plus(sph) : cut_phase_minus(sph);
       double Mp[10];
+#pragma unroll
       for (int k = 0; k < 10; ++k) Mp[k] = dp[(long long)cut_f_M(si, k) * ncut + e];
       side_weights(L, si == 0 ? 1.0 : -1.0, gr, Mp, ph.lam[f] * sv, ph.mu[f] * sv, w[si]);
       const SideW& W = w[si];
       lam += W.V * W.lam;
       mu += W.V * W.mu;
+#pragma unroll
       for (int b = 0; b < 4; ++b)
+#pragma unroll
         for (int x = 0; x < 3; ++x) {
           const double v = W.P * gr[b][x] + W.m[b] * W.gam[x];
           l[b][x] += W.lam * v;
@@ -526,16 +543,52 @@ __global__ void __launch_bounds__(128) k_cut_elements(const int* __restrict__ ip
         }
     }
     double* R = el + ((long long)(e >> 5) * kEl) * 32 + (e & 31);
-    R[0] = lam;
-    R[32] = mu;
-    for (int b = 0; b < 4; ++b)
-      for (int x = 0; x < 3; ++x) {
-        R[32 * (kElL + 3 * b + x)] = dsc[b][x] * l[b][x];
-        for (int y = 0; y < 3; ++y) R[32 * (kElP + 9 * b + 3 * x + y)] = dsc[b][x] * p[b][y];
-      }
-    int k = 0;
+    const auto put = [&](int k, double v) { R[32 * k] = v; };
+    put(0, lam);
+    put(1, mu);
+#pragma unroll
+    for (int i = 0; i < 12; ++i) put(kElL + i, dsc[i / 3][i % 3] * l[i / 3][i % 3]);
+#pragma unroll
     for (int i = 0; i < 12; ++i)
-      for (int j = i; j < 12; ++j, ++k) R[32 * (kElK + k)] = cut_element_entry(12 + i, 12 + j, w, gr, dsc);
+#pragma unroll
+      for (int y = 0; y < 3; ++y) put(kElP + 3 * i + y, dsc[i / 3][i % 3] * p[i / 3][y]);
+    // K's upper triangle row by row: rows 3 a + x, columns 3 b + y with b >= a
+    int k = kElK;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      double B[4][3][3];
+#pragma unroll
+      for (int b = a; b < 4; ++b) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+#pragma unroll
+          for (int y = 0; y < 3; ++y) B[b][x][y] = 0.0;
+#pragma unroll
+        for (int si = 0; si < 2; ++si) {
+          const SideW& W = w[si];
+          double A[3][3];
+#pragma unroll
+          for (int y = 0; y < 3; ++y) {
+            const double h = W.Q * gr[b][y] + W.R[b] * W.gam[y];
+            const double c = W.R[a] * gr[b][y] + W.M[a][b] * W.gam[y];
+#pragma unroll
+            for (int x = 0; x < 3; ++x) A[x][y] = gr[a][x] * h + W.gam[x] * c;
+          }
+          const double mt = W.mu * (A[0][0] + A[1][1] + A[2][2]);
+#pragma unroll
+          for (int x = 0; x < 3; ++x)
+#pragma unroll
+            for (int y = 0; y < 3; ++y) B[b][x][y] += W.lam * A[x][y] + W.mu * A[y][x] + (x == y ? mt : 0.0);
+        }
+      }
+#pragma unroll
+      for (int x = 0; x < 3; ++x)
+#pragma unroll
+        for (int b = a; b < 4; ++b)
+#pragma unroll
+          for (int y = 0; y < 3; ++y)
+            if (b > a || y >= x) put(k++, dsc[a][x] * dsc[b][y] * B[b][x][y]);
+    }
   }
 }
 
@@ -676,20 +729,6 @@ cudaError_t launch_finish_scaling(const double* D, double* isd, float* isf, int 
   if (nX == 0) return cudaSuccess;
   const long long n = 3LL * nX;
   k_finish_scaling<<<(int)((n + 255) / 256), 256, 0, s>>>(D, isd, isf, n);
-  return cudaGetLastError();
-}
-
-__global__ void k_to_float(const double* __restrict__ a, float* __restrict__ b, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x)
-    b[i] = (float)a[i];
-}
-
-cudaError_t launch_cut_to_float(const double* dp, float* fp, long long count, cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  long long nb = (count + 255) / 256;
-  if (nb > 65535LL * 16) nb = 65535LL * 16;
-  k_to_float<<<(int)nb, 256, 0, s>>>(dp, fp, count);
   return cudaGetLastError();
 }
 

@@ -21,7 +21,6 @@ namespace xfft {
 struct CutData {
   const int* ip;
   const double* dp;
-  const float* fp;
   int ncut;
   // per cut tet, for the apply kernels: the four node ids and enriched ids (int4 each) and a
   // record of kRec reals (FP32 and FP64 copies; layout below)
@@ -86,7 +85,6 @@ cudaError_t launch_block_inverse(const double* D, const double* Doff, const doub
                                  float* b32, int nX, int* bad, cudaStream_t s);
 cudaError_t launch_finish_scaling(const double* D, double* isd, float* isf, int nX,
                                   cudaStream_t s);
-cudaError_t launch_cut_to_float(const double* dp, float* fp, long long count, cudaStream_t s);
 // apply records and node / enriched id quadruples of the cut tets (needs isD, phases, scale)
 cudaError_t launch_cut_records(CutData cd, const double* isD, int nX, GridDev g, PhaseDev ph,
                                const float* scale, int4* n4, int4* e4, double* r64, float* r32,
