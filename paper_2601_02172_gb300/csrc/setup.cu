@@ -612,6 +612,7 @@ __global__ void k_cut_records(const int* __restrict__ ip, const double* __restri
     const int t = ip[9 * ncut + e];
     const int sph = ip[kCutFieldPhases * ncut + e];
     int nd[4], ej[4];
+#pragma unroll
     for (int a = 0; a < 4; ++a) {
       nd[a] = ip[a * ncut + e];
       ej[a] = ip[(4 + a) * ncut + e];
@@ -622,44 +623,59 @@ __global__ void k_cut_records(const int* __restrict__ ip, const double* __restri
     tet_grads<double>(t, ih, gr);
     const double sv = scale ? (double)scale[vox] : 1.0;
     double R[kRec];
-    for (int k = 0; k < kRec; ++k) R[k] = 0.0;
+#pragma unroll
     for (int a = 0; a < 4; ++a)
+#pragma unroll
       for (int x = 0; x < 3; ++x) R[3 * a + x] = isD[(long long)x * nX + ej[a]];
     double L[4];
+#pragma unroll
     for (int b = 0; b < 4; ++b) L[b] = dp[(long long)cut_f_L(b) * ncut + e];
+#pragma unroll
     for (int si = 0; si < 2; ++si) {
-      double* S = R + kRecSide + kRecSideLen * si;
+      const int S = kRecSide + kRecSideLen * si;
       const double sg = si == 0 ? 1.0 : -1.0;
       double M[10], m[4], c[4];
+#pragma unroll
       for (int k = 0; k < 10; ++k) M[k] = dp[(long long)cut_f_M(si, k) * ncut + e];
+#pragma unroll
       for (int b = 0; b < 4; ++b) {
         m[b] = dp[(long long)cut_f_m(si, b) * ncut + e];
         c[b] = fabs(L[b]) - sg * L[b];
       }
       double V = 0.0, mc = 0.0, cMc = 0.0, gam[3] = {0.0, 0.0, 0.0};
+#pragma unroll
       for (int b = 0; b < 4; ++b) {
         double P = 0.0;
+#pragma unroll
         for (int cc = 0; cc < 4; ++cc) P += M[midx(b, cc)] * c[cc];
-        S[14 + b] = P;
-        S[10 + b] = m[b];
+        R[S + 14 + b] = P;
+        R[S + 10 + b] = m[b];
         V += m[b];
         mc += m[b] * c[b];
         cMc += P * c[b];
+#pragma unroll
         for (int x = 0; x < 3; ++x) gam[x] += c[b] * gr[b][x];
       }
-      for (int k = 0; k < 10; ++k) S[k] = M[k];
-      for (int x = 0; x < 3; ++x) S[18 + x] = gam[x];
+#pragma unroll
+      for (int k = 0; k < 10; ++k) R[S + k] = M[k];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) R[S + 18 + x] = gam[x];
       const int p = si == 0 ? cut_phase_plus(sph) : cut_phase_minus(sph);
-      S[21] = ph.lam[p] * sv;
-      S[22] = ph.mu[p] * sv;
-      S[23] = V;
-      S[24] = mc;
-      S[25] = cMc;
+      R[S + 21] = ph.lam[p] * sv;
+      R[S + 22] = ph.mu[p] * sv;
+      R[S + 23] = V;
+      R[S + 24] = mc;
+      R[S + 25] = cMc;
+      R[S + 26] = R[S + 27] = 0.0;
     }
-    for (int k = 0; k < kRec; ++k) {
-      r64[(long long)e * kRec + k] = R[k];
-      r32[(long long)e * kRec + k] = (float)R[k];
-    }
+    // 16-byte stores: rows are 544 and 272 bytes apart, so every narrower one costs a sector as well
+    double2* o64 = reinterpret_cast<double2*>(r64 + (long long)e * kRec);
+    float4* o32 = reinterpret_cast<float4*>(r32 + (long long)e * kRec);
+#pragma unroll
+    for (int k = 0; k < kRec / 2; ++k) o64[k] = make_double2(R[2 * k], R[2 * k + 1]);
+#pragma unroll
+    for (int k = 0; k < kRec / 4; ++k)
+      o32[k] = make_float4((float)R[4 * k], (float)R[4 * k + 1], (float)R[4 * k + 2], (float)R[4 * k + 3]);
   }
 }
 
