@@ -280,6 +280,9 @@ XFFT_APPLY_INST_NPH(, double, 2)
 XFFT_APPLY_INST_NPH(, dw, 2)
 
 // ---------------------------------------------------------------- per-voxel average stress
+// Bound by the FP64 pipe.  Voxels of one phase need the stress of one summed strain (60 FP64 operations
+// instead of 165), cut tets one strain per side from the side's first moments instead of one per vertex:
+// 256^3 with 4.1 million cut tets 10.4 -> 7.5 ms, 200 x 160 x 144 2.6 -> 1.9 ms.
 __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyArgs a,
                                      double* __restrict__ out) {
   const int rhs = blockIdx.y;
@@ -309,19 +312,44 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
       lms[p] = a.ph.lam[p] * sv;
       mus[p] = a.ph.mu[p] * sv;
     }
-    // the voxel's edge differences (with eps_bar) and tension sums, as in the stencil
-    double D[12][3], Te[12][3], sg[6] = {0, 0, 0, 0, 0, 0};
+    double sg[6] = {0, 0, 0, 0, 0, 0};
+    const unsigned code = a.code[v];
+    const bool one = code == 0u || code == 0x555u || code == 0xfffu;
+    if (__all_sync(__activemask(), one)) {
+      // one phase (most warps): the stress of the six tets' summed gradient, in which the voxel's
+      // first and last path edges count twice and the middle ones once (a third of the FP64
+      // operations, which bound this kernel)
+      double H[3][3];  // sum over the tets of d u_x / d x_ax
 #pragma unroll
-    for (int ax = 0; ax < 3; ++ax)
+      for (int ax = 0; ax < 3; ++ax)
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (!(c & (1 << ax))) {
-#pragma unroll
-          for (int x = 0; x < 3; ++x)
-            D[cube_edge(c, ax)][x] = (uu[c | (1 << ax)][x] - uu[c][x]) * ih[ax] + sym_at(E, x, ax);
+        for (int x = 0; x < 3; ++x) {
+          const int e = 1 << ax, m1 = ax == 0 ? 2 : 1, m2 = ax == 2 ? 2 : 4;  // the other two axes' corners
+          const double ends = (uu[e][x] - uu[0][x]) + (uu[7][x] - uu[7 ^ e][x]);
+          const double mid = (uu[e | m1][x] - uu[m1][x]) + (uu[e | m2][x] - uu[m2][x]);
+          H[ax][x] = (2.0 * ends + mid) * ih[ax];
         }
-    voxel_tets<double, kMaxPhases>(D, Te, a.code[v], lms, mus);
-    voxel_stress_sums(Te, sg);
+      const int p = code == 0u ? 0 : code == 0xfffu ? 2 : 1;
+      const double lam = p == 0 ? lms[0] : p == 1 ? lms[1] : lms[2], mu = p == 0 ? mus[0] : p == 1 ? mus[1] : mus[2];
+      const double e6[6] = {H[0][0] + 6.0 * E[0], H[1][1] + 6.0 * E[1], H[2][2] + 6.0 * E[2],
+                            0.5 * (H[1][2] + H[2][1]) + 6.0 * E[3], 0.5 * (H[0][2] + H[2][0]) + 6.0 * E[4],
+                            0.5 * (H[0][1] + H[1][0]) + 6.0 * E[5]};
+      iso_stress(e6, lam, mu, sg);
+    } else {
+      // the voxel's edge differences (with eps_bar) and tension sums, as in the stencil
+      double D[12][3], Te[12][3];
+#pragma unroll
+      for (int ax = 0; ax < 3; ++ax)
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+          if (!(c & (1 << ax))) {
+#pragma unroll
+            for (int x = 0; x < 3; ++x)
+              D[cube_edge(c, ax)][x] = (uu[c | (1 << ax)][x] - uu[c][x]) * ih[ax] + sym_at(E, x, ax);
+          }
+      voxel_tets<double, kMaxPhases>(D, Te, code, lms, mus);
+      voxel_stress_sums(Te, sg);
+    }
 #pragma unroll
     for (int x = 0; x < 6; ++x) sg[x] *= g.vol_tet;
     const double r2 = 1.41421356237309504880;
@@ -388,23 +416,29 @@ __global__ void k_voxel_stress_cut(const double* __restrict__ u, const double* _
       const double s = si == 0 ? 1.0 : -1.0;
       const int ph = si == 0 ? cut_phase_plus(sph) : cut_phase_minus(sph);
       const double lam = a.ph.lam[ph] * sv, mu = a.ph.mu[ph] * sv;
-      double c[4], gam[3] = {0, 0, 0};
+      // int over the side of C (es + sum_b N_b (c_b ew + sym(w_b (x) gamma))) from its moments m_b
+      double gam[3] = {0, 0, 0}, W[3] = {0, 0, 0}, V = 0.0, mc = 0.0;
+#pragma unroll
       for (int b = 0; b < 4; ++b) {
-        c[b] = fabs(L[b]) - s * L[b];
-        for (int x = 0; x < 3; ++x) gam[x] += c[b] * gr[b][x];
-      }
-      for (int b = 0; b < 4; ++b) {
+        const double c = fabs(L[b]) - s * L[b];
         const double mb = cd.dp[(long long)cut_f_m(si, b) * ncut + e];
-        const double* wb = ws[b];
-        double eb[6] = {es[0] + c[b] * ew[0] + wb[0] * gam[0], es[1] + c[b] * ew[1] + wb[1] * gam[1],
-                        es[2] + c[b] * ew[2] + wb[2] * gam[2],
-                        es[3] + c[b] * ew[3] + 0.5 * (wb[1] * gam[2] + wb[2] * gam[1]),
-                        es[4] + c[b] * ew[4] + 0.5 * (wb[0] * gam[2] + wb[2] * gam[0]),
-                        es[5] + c[b] * ew[5] + 0.5 * (wb[0] * gam[1] + wb[1] * gam[0])};
-        double sb[6];
-        iso_stress(eb, lam, mu, sb);
-        for (int k = 0; k < 6; ++k) tot[k] += mb * sb[k];
+        V += mb;
+        mc += mb * c;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+          gam[x] += c * gr[b][x];
+          W[x] += mb * ws[b][x];
+        }
       }
+      const double eb[6] = {V * es[0] + mc * ew[0] + W[0] * gam[0], V * es[1] + mc * ew[1] + W[1] * gam[1],
+                            V * es[2] + mc * ew[2] + W[2] * gam[2],
+                            V * es[3] + mc * ew[3] + 0.5 * (W[1] * gam[2] + W[2] * gam[1]),
+                            V * es[4] + mc * ew[4] + 0.5 * (W[0] * gam[2] + W[2] * gam[0]),
+                            V * es[5] + mc * ew[5] + 0.5 * (W[0] * gam[1] + W[1] * gam[0])};
+      double sb[6];
+      iso_stress(eb, lam, mu, sb);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) tot[k] += sb[k];
     }
     const double r2 = 1.41421356237309504880;
     double* o = out + (long long)rhs * 6 * N;
