@@ -490,6 +490,7 @@ static void free_work(xfft_ctx* c) {
   dfree(c, c->eps_d);
   dfree(c, c->sig_keep);
   dfree(c, c->partials);
+  c->partials_count = 0;
   dfree(c, c->red_out);
   dfree(c, c->bbpart);
   c->cap_rhs = 0;
@@ -729,9 +730,33 @@ static int nparts_of(const xfft_ctx* c) {
                   std::max(precondition_blocks(c->fft, c->nX, true), precondition_blocks(c->fft, c->nX, false)));
 }
 
+// doubles of the partial-sum buffer that calls of up to n_rhs right-hand sides index.  It depends on
+// the number of cut tets as well: two microstructures with the same enriched nodes (the same stride)
+// may differ in it.
+static size_t partials_needed(const xfft_ctx* c, int n_rhs) {
+  const int ng = grad_blocks_uncut(c->g) + grad_blocks_cut(c->ncut);
+  return std::max((size_t)n_rhs * 7 * nparts_of(c), (size_t)kGradValues * ng);
+}
+
+// refuses a launch whose partial sums the buffer does not hold (every entry point's ensure_work
+// provides for it)
+static xfft_status partials_fit(const xfft_ctx* c, int n_rhs) {
+  return c->partials_count >= partials_needed(c, n_rhs) ? XFFT_OK
+                                                        : fail(XFFT_ESTATE, "partial-sum buffer too small");
+}
+
 static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   const long long stride = stride_of(c);
-  if (c->cap_rhs >= n_rhs && c->cap_stride == stride && c->cap_prec == prec) return XFFT_OK;
+  if (c->cap_rhs >= n_rhs && c->cap_stride == stride && c->cap_prec == prec) {
+    const size_t need = partials_needed(c, c->cap_rhs);
+    if (c->partials_count >= need) return XFFT_OK;
+    drop_graphs(c);  // they hold the buffer's address
+    dfree(c, c->partials);
+    c->partials_count = 0;
+    CU(dalloc(c, &c->partials, need));
+    c->partials_count = need;
+    return XFFT_OK;
+  }
   Recycle recycle(c);
   free_work(c);
   const size_t tot = (size_t)n_rhs * stride;
@@ -749,10 +774,9 @@ static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   CU(dalloc(c, &c->outer_mask, 64));
   CU(dalloc(c, &c->eps_d, 6 * 64));
   CU(dalloc(c, &c->sig_keep, 6 * 64));
-  const int ng = grad_blocks_uncut(c->g) + grad_blocks_cut(c->ncut);
-  const int nparts = nparts_of(c);
-  c->partials_count = std::max((size_t)n_rhs * 7 * nparts, (size_t)kGradValues * ng);
-  CU(dalloc(c, &c->partials, c->partials_count));
+  const size_t need = partials_needed(c, n_rhs);
+  CU(dalloc(c, &c->partials, need));
+  c->partials_count = need;
   CU(dalloc(c, &c->red_out, 64));
   if (bb_euclid(c)) CU(dalloc(c, &c->bbpart, (size_t)n_rhs * 2 * kBBParts));
   c->cap_rhs = n_rhs;
@@ -830,6 +854,7 @@ static xfft_status do_apply(xfft_ctx* c, const T* d, T* q, const double* eps_dev
                             const T* fz = nullptr, T* fdnew = nullptr, T* fu = nullptr, int parity = 0,
                             int want_sig = -1, bool sig_add = false) {
   static_assert(std::is_same<typename Store<A>::type, T>::value, "arithmetic/storage mismatch");
+  if (const xfft_status fit = partials_fit(c, n_rhs)) return fit;
   ApplyArgs a = apply_args(c, eps_dev, active);
   a.fz = fz;
   a.fdnew = fdnew;
@@ -877,6 +902,7 @@ template <typename T>
 static xfft_status do_prec(xfft_ctx* c, T* f, T* z, int n_rhs, const int* active, int fin_mode,
                            double tol, int crit, int maxit, int set_rel = 0, const T* qfuse = nullptr,
                            int parity = 0) {
+  if (const xfft_status fit = partials_fit(c, n_rhs)) return fit;
   const int nparts = nparts_of(c);
   {
     const int kp = sizeof(T) == 8 ? XFFT_PROF_PREC_F64 : XFFT_PROF_PREC_F32;
@@ -1842,6 +1868,7 @@ extern "C" xfft_status xfft_grad_phases(xfft_ctx* c, const double dL_dCeff[36], 
   if (!c || !dL_dCeff || !dL_dlame) return fail(XFFT_EINVAL, "NULL argument");
   if (!c->have_micro || !c->have6) return fail(XFFT_ESTATE, "xfft_effective_stiffness first");
   TRY(ensure_work(c, 6, c->cap_prec >= 0 ? c->cap_prec : c->opt.precision));
+  TRY(partials_fit(c, 6));
   const GridDev& g = c->g;
   cudaStream_t s = c->stream;
   GradArgs a;

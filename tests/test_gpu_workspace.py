@@ -1,0 +1,68 @@
+"""What a context keeps between calls: the workspace over microstructures and numbers of right-hand
+sides, against contexts that have seen one call only."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def xf():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2601_02172_gb300 as pkg
+    return pkg
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+LM, LP = synth.lame_from_E_nu(10.0, 0.25), synth.lame_from_E_nu(1.0, 0.3)
+
+
+def _equal_enriched_nodes(n=(60, 60, 80)):
+    """Two level sets with the same number of enriched nodes and different numbers of cut tets: 1280
+    isolated negative nodes (15 enriched nodes, 24 cut tets each) and a slab of negative planes (its four
+    bounding node planes)."""
+    few = np.ones(n)
+    few.reshape(-1)[np.ravel_multi_index(
+        [v.ravel()[:1280] for v in np.meshgrid(*[np.arange(0, m - 2, 3) for m in n], indexing="ij")], n)] = -0.7
+    many = np.ones(n)
+    many[20:40] = -0.7
+    return n, few, many
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_more_cut_tets_on_the_same_enriched_nodes(xf, precision):
+    """The partial sums grow with the cut tets while the vectors stay as long as they were.  Applies
+    agree to rounding (1e-12, FP32 2e-5), stresses to ten times the solver's tolerance, gradients (of first
+    order in the fields' error, in part FP32) to a few FP32 roundings."""
+    n, few, many = _equal_enriched_nodes()
+    kept, fresh = xf.Solver(n, precision=precision), xf.Solver(n, precision=precision)
+    kept.set_microstructure(few, LM, LP)
+    fresh.set_microstructure(many, LM, LP)
+    rng = np.random.default_rng(3)
+    d, eps = rng.normal(size=(8, kept.stride)), rng.normal(size=(8, 6))
+    kept.apply(d, eps)
+    kept.effective_stiffness()
+    few_cut, nX = kept.num_cut_tets, kept.num_enriched
+    kept.set_microstructure(many, LM, LP)
+    assert kept.num_enriched == nX and kept.num_cut_tets > 1.5 * few_cut
+    for prec, tol in (("fp64", 1e-12), ("fp32", 2e-5)):
+        (q, sig), (q0, sig0) = (s.apply(d, eps, precision=prec) for s in (kept, fresh))
+        assert _rel(q, q0) < tol and _rel(sig, sig0) < tol
+    (a, b) = (s.solve(eps, u=False)["mean_stress"] for s in (kept, fresh))
+    assert _rel(a, b) < 1e-9
+    (C, st), (C0, st0) = (s.effective_stiffness() for s in (kept, fresh))
+    assert st["converged"] and st0["converged"] and _rel(C, C0) < 1e-9
+    G = rng.normal(size=(6, 6))
+    for x, x0 in zip(kept.grad(G), fresh.grad(G)):
+        assert _rel(x, x0) < 1e-6
+    kept.close()
+    fresh.close()
