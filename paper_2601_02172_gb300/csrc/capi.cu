@@ -777,7 +777,7 @@ static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
   const size_t need = partials_needed(c, n_rhs);
   CU(dalloc(c, &c->partials, need));
   c->partials_count = need;
-  CU(dalloc(c, &c->red_out, 64));
+  CU(dalloc(c, &c->red_out, std::max(7 * 64, kGradValues)));  // seven sums of up to 64 right-hand sides
   if (bb_euclid(c)) CU(dalloc(c, &c->bbpart, (size_t)n_rhs * 2 * kBBParts));
   c->cap_rhs = n_rhs;
   c->cap_stride = stride;

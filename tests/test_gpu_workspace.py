@@ -66,3 +66,23 @@ def test_more_cut_tets_on_the_same_enriched_nodes(xf, precision):
         assert _rel(x, x0) < 1e-6
     kept.close()
     fresh.close()
+
+
+def test_stress_integrals_of_sixty_four_right_hand_sides(xf):
+    """The reduced sums of an apply (seven per right-hand side) at the largest number of right-hand
+    sides, against the same vectors in groups of eight; the solve that follows is that of a fresh context."""
+    n = (12, 10, 8)
+    L = synth.sphere_levelset(n, (0.5, 0.45, 0.55), 0.3)
+    s, fresh = xf.Solver(n), xf.Solver(n)
+    for v in (s, fresh):
+        v.set_microstructure(L, LM, LP)
+    rng = np.random.default_rng(5)
+    d, eps = rng.normal(size=(64, s.stride)), rng.normal(size=(64, 6))
+    q, sig = s.apply(d, eps)
+    for r in range(0, 64, 8):
+        q8, sig8 = fresh.apply(d[r:r + 8], eps[r:r + 8])
+        assert _rel(q[r:r + 8], q8) < 1e-12 and _rel(sig[r:r + 8], sig8) < 1e-12
+    (C, _), (C0, _) = s.effective_stiffness(), fresh.effective_stiffness()
+    assert _rel(C, C0) < 1e-9
+    s.close()
+    fresh.close()
