@@ -293,8 +293,11 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
   double ih[3];
   for (int k = 0; k < 3; ++k) ih[k] = 1.0 / g.h[k];
   const double ivox = 1.0 / (6.0 * g.vol_tet);
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
-       v += (long long)gridDim.x * blockDim.x) {
+  // whole warps stay in the loop for the vote below; lanes past the end repeat the last voxel
+  for (long long w0 = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); w0 < g.N;
+       w0 += (long long)gridDim.x * blockDim.x) {
+    const bool inside = w0 + (threadIdx.x & 31) < g.N;
+    const long long v = inside ? w0 + (threadIdx.x & 31) : g.N - 1;
     const int k = (int)(v % g.n2);
     const int j = (int)((v / g.n2) % g.n1);
     const int i = (int)(v / ((long long)g.n1 * g.n2));
@@ -315,7 +318,7 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
     double sg[6] = {0, 0, 0, 0, 0, 0};
     const unsigned code = a.code[v];
     const bool one = code == 0u || code == 0x555u || code == 0xfffu;
-    if (__all_sync(__activemask(), one)) {
+    if (__all_sync(0xffffffffu, one)) {
       // one phase (most warps): the stress of the six tets' summed gradient, in which the voxel's
       // first and last path edges count twice and the middle ones once (a third of the FP64
       // operations, which bound this kernel)
@@ -350,6 +353,7 @@ __global__ void k_voxel_stress_uncut(const double* __restrict__ u, const ApplyAr
       voxel_tets<double, kMaxPhases>(D, Te, code, lms, mus);
       voxel_stress_sums(Te, sg);
     }
+    if (!inside) continue;
 #pragma unroll
     for (int x = 0; x < 6; ++x) sg[x] *= g.vol_tet;
     const double r2 = 1.41421356237309504880;

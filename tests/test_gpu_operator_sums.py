@@ -1,0 +1,42 @@
+"""Sums over voxels at the edges of the kernels that form them."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import XFEM
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def xf():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2601_02172_gb300 as pkg
+    return pkg
+
+
+def _rel(a, b):
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+LM, LP = synth.lame_from_E_nu(10.0, 0.25), synth.lame_from_E_nu(1.0, 0.3)
+
+
+@pytest.mark.parametrize("n", [(6, 6, 6), (10, 6, 6), (10, 10, 6), (8, 8, 4)])
+def test_voxel_stress_of_a_partly_filled_warp(xf, n):
+    """Numbers of voxels that leave 24, 8, 24 and 0 lanes of the last warp, each with one-phase and with
+    cut voxels, against the oracle's stress of the same displacements (linear in them: rounding only)."""
+    L = synth.sphere_levelset(n, (0.45, 0.5, 0.55), 0.3)
+    s = xf.Solver(n)
+    s.set_microstructure(L, LM, LP)
+    o = XFEM(L, n, lame_minus=LM, lame_plus=LP)
+    eps = np.random.default_rng(1).normal(size=(2, 6))
+    out = s.solve(eps, voxel_stress=True)
+    for r in range(2):
+        u = np.concatenate([out["u_std"][r].ravel(), (out["u_enr"][r] / o.Dinvsqrt.T).ravel()])
+        assert _rel(out["voxel_stress"][r], o.voxel_stress(u, eps[r]).T) < 1e-12
+    s.close()
