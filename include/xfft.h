@@ -304,6 +304,11 @@ xfft_status xfft_profile_read(xfft_ctx* ctx, double ms[16], long long launches[1
  * is looked up once, by the first xfft_set_microstructure (or xfft_apply_noalloc) on that
  * device; a first lookup attempted while the context's stream is being captured returns
  * XFFT_ESTATE instead.
+ * The call may be captured into a CUDA graph; the graph reads the microstructure's buffers and can
+ * be replayed until the next xfft_set_microstructure or xfft_destroy, whatever other calls the
+ * context serves in between.  (An FP64 context's eager applies read reduced cut-tet records where
+ * device memory and max_device_bytes have room for them; they may be given up for a later call's
+ * buffers, so a captured apply reads the moment records and takes the longer of the two ways.)
  * Every call shares the one scratch array: calls that overlap on the GPU (other streams,
  * other threads, other contexts on the same device) race and must be serialised by the
  * caller.  The context must exist with its microstructure set (those calls do allocate). */

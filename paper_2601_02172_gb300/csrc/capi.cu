@@ -228,7 +228,8 @@ static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes) {
         continue;
       }
     }
-    // the reduced element records are a speed-up that gives way to what a call cannot do without
+    // the reduced element records are a speed-up that gives way to what a call cannot do without;
+    // nothing else holds their address (an apply captured by the caller does not read them)
     if (e != cudaErrorMemoryAllocation || !c->cut_el) return e;
     cudaGetLastError();
     cudaStreamSynchronize(c->stream);
@@ -2148,8 +2149,14 @@ extern "C" xfft_status xfft_apply_noalloc(xfft_ctx* c, int n_rhs, const double* 
   // and the cut-tet kernel's fit the scratch for every grid that it admits
   if (apply_uncut_blocks(c->g) + apply_cut_blocks(c->ncut) > XFFT_NOALLOC_MAX_PARTS)
     return fail(XFFT_EINVAL, "grid too large for the fixed scratch of xfft_apply_noalloc");
+  // A captured apply is replayed after calls that may have given the reduced element records up for
+  // memory (dalloc_bytes): it takes the moment records, which live until the next microstructure.
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (c->stream) CU(cudaStreamIsCapturing(c->stream, &cs));
+  CutData cd = cutdata(c);
+  if (cs != cudaStreamCaptureStatusNone) cd.el = nullptr;
   const int tile_blocks = apply_tile_blocks(c->g, n_rhs);
-  const int nparts = tile_blocks + cut_blocks_of(c, false);
+  const int nparts = tile_blocks + (cd.el ? apply_cut_el_blocks(c->ncut) : apply_cut_blocks(c->ncut));
   if (nparts > XFFT_NOALLOC_MAX_PARTS) return fail(XFFT_EINVAL, "partial sums exceed the fixed scratch");
   double* scratch = nullptr;
   TRY(noalloc_scratch(&scratch, c->stream));
@@ -2173,7 +2180,7 @@ extern "C" xfft_status xfft_apply_noalloc(xfft_ctx* c, int n_rhs, const double* 
   a.fdnew = nullptr;
   a.fu = nullptr;
   a.st = nullptr;
-  CU(launch_apply<double>(d, q, c->isD, cutdata(c), a, n_rhs, c->stream));
+  CU(launch_apply<double>(d, q, c->isD, cd, a, n_rhs, c->stream));
   if (dAd_sig) CU(launch_reduce_partials(scratch, 7 * n_rhs, nparts, nparts, dAd_sig, c->stream));
   return XFFT_OK;
 }

@@ -86,3 +86,55 @@ def test_stress_integrals_of_sixty_four_right_hand_sides(xf):
     assert _rel(C, C0) < 1e-9
     s.close()
     fresh.close()
+
+
+def test_captured_apply_outlives_the_reduced_records(xf):
+    """An FP64 apply captured by the caller, replayed before and after a call whose buffers push the
+    reduced cut-tet records out of the memory cap, over caps a quarter of the records apart: the replays
+    agree with the eager apply (1e-12) and with each other, also once the freed memory holds NaN."""
+    import torch
+    n = (16, 12, 10)
+    L = synth.sphere_levelset(n, (0.5, 0.45, 0.55), 0.3)
+    ref = xf.Solver(n)
+    ref.set_microstructure(L, LM, LP)
+    ncut = ref.num_cut_tets
+    big = np.random.default_rng(2).normal(size=(24, ref.stride))
+    qb, sb = ref.apply(big)
+    ref.close()
+    d = torch.from_numpy(big[:2]).cuda()
+    served = refused = 0
+    for cap in range(4 << 20, 48 << 20, 256 * ncut):
+        st = torch.cuda.Stream()
+        s = xf.Solver(n, max_device_bytes=cap, stream=st)
+        try:
+            s.set_microstructure(L, LM, LP)
+        except xf.XfftError as e:
+            assert e.status == xf.capi.XFFT_ENOMEM
+            s.close()
+            continue
+        q = torch.full_like(d, float("nan"))
+        out = torch.full((2, 7), float("nan"), dtype=torch.float64, device="cuda")
+        s.apply_noalloc(d, q, out)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=st):
+            s.apply_noalloc(d, q, out)
+        for after in (False, True):
+            if after:
+                try:
+                    assert _rel(s.apply(big)[0], qb) < 1e-12
+                    served += 1
+                except xf.XfftError as e:
+                    assert e.status == xf.capi.XFFT_ENOMEM
+                    refused += 1
+                junk = [torch.full((1024 * ncut // 16,), float("nan"), dtype=torch.float64, device="cuda")
+                        for _ in range(4)]
+            q.fill_(float("nan"))
+            out.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            assert _rel(q.cpu().numpy(), qb[:2]) < 1e-12, (cap, after)
+            assert _rel(out.cpu().numpy()[:, 1:], sb[:2]) < 1e-12, (cap, after)
+        del junk, graph
+        s.close()
+    assert served >= 4 and refused >= 1
