@@ -210,6 +210,10 @@ FftPlan* fft_plan_create(const GridDev& g, bool dbl, cudaError_t* err) {
     delete p;
     return nullptr;
   }
+  if ((*err = lines_opt_in<float>()) != cudaSuccess || (*err = lines_opt_in<double>()) != cudaSuccess) {
+    delete p;
+    return nullptr;
+  }
   // tables: twiddles exp(-2 pi i k / n) and Green phases per axis
   const int n[3] = {g.n0, g.n1, g.n2};
   size_t tot2d = 0;

@@ -659,7 +659,10 @@ struct LineGrid {
 };
 bool line_grid(LineGrid& g, int n0, int n1, int n2, bool dbl);  // false for an unsupported length (fft.cu)
 
-// launchers of one precision (instantiated in fft_lines_f32.cu and fft_lines_f64.cu)
+// launchers of one precision (instantiated in fft_lines_f32.cu and fft_lines_f64.cu); lines_opt_in at the
+// creation of a plan, for the current device
+template <typename T>
+cudaError_t lines_opt_in();
 template <typename T>
 cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec, long long stride, long long sstride,
                                const int* active, const void* const* tw, const T* table, unsigned long long* units,

@@ -8,28 +8,43 @@
 namespace xfft {
 namespace lines {
 
+// The most dynamic shared memory that a launch below asks for (column_bits; the z passes stay at 64 KB).
+constexpr size_t kLineShared = 200 * 1024;
+
 // Columns per block (2^lb) of the y and x passes: 128 bytes of every plane crossed, fewer where a
 // block's lines would pass 100 KB of shared memory (two blocks per SM) or the launch would not give
 // every SM two blocks; never below 4 (32-byte sectors) unless shared memory asks for it.
 inline int column_bits(size_t line_bytes, size_t csize, long long cols, int n_rhs) {
   int lb = csize == 8 ? 4 : 3;
   while (lb > 2 && ((line_bytes << lb) > 100 * 1024 || ((cols >> lb) + 1) * n_rhs < 2 * 152)) --lb;
-  while (lb > 0 && (line_bytes << lb) > 200 * 1024) --lb;
+  while (lb > 0 && (line_bytes << lb) > kLineShared) --lb;
   return lb;
 }
 inline int column_threads(const LinePlan& p, int lb) {
   const int items = (p.n / std::min(p.R1, p.RL)) << lb;
   return std::min(kLineThreads, std::max(32, (items + 31) / 32 * 32));
 }
-template <typename K>
-cudaError_t opt_in(K kernel, size_t bytes) {
-  if (bytes <= 48 * 1024) return cudaSuccess;
-  return cudaFuncSetAttribute((const void*)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 inline int max_radix(const LinePlan& p) { return std::max(p.R1, std::max(p.RM, p.RL)); }
 
 }  // namespace lines
+
+// All lengths share the kernels of a precision and radix class, and the opt-in to more than 48 KB of
+// shared memory belongs to the kernel, not to a launch: every plan gives the same, largest one, so that
+// no launch of another grid (another context in another thread, another node of a graph) finds it lowered.
+template <typename T>
+cudaError_t lines_opt_in() {
+  using namespace lines;
+  const void* const kernels[] = {
+      (const void*)k_line_z_fwd<T, 12>,    (const void*)k_line_z_fwd<T, 16>,    (const void*)k_line_z_inv<T, 12>,
+      (const void*)k_line_z_inv<T, 16>,    (const void*)k_line_y<T, 12, false>, (const void*)k_line_y<T, 16, false>,
+      (const void*)k_line_y<T, 12, true>,  (const void*)k_line_y<T, 16, true>,  (const void*)k_line_x<T, 12>,
+      (const void*)k_line_x<T, 16>};
+  for (const void* k : kernels) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 template <typename T>
 cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long long stride, long long sstride,
@@ -49,12 +64,10 @@ cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long
   const int tz = std::min(kLineThreads, std::max(32, (nz + 31) / 32 * 32));
   const auto fz = max_radix(pz) > 12 ? k_line_z_fwd<T, 16> : k_line_z_fwd<T, 12>;
   const auto iz = max_radix(pz) > 12 ? k_line_z_inv<T, 16> : k_line_z_inv<T, 12>;
-  cudaError_t e = opt_in(fz, smz);
-  if (e == cudaSuccess) e = opt_in(iz, smz);
-  if (e != cudaSuccess) return e;
   fz<<<dim3(g.zblocks, n_rhs), tz, smz, s>>>(f, spec, stride, sstride, pz, g.rp, rows, active, tw2, units,
                                                           q, st);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
 
   const int ycols = 3 * g.n0 * g.K2;
   const size_t ly = sizeof(C) * g.n1;
@@ -63,9 +76,6 @@ cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long
   const bool big_y = max_radix(g.ax[1]) > 12;
   const auto fy = big_y ? k_line_y<T, 16, false> : k_line_y<T, 12, false>;
   const auto iy = big_y ? k_line_y<T, 16, true> : k_line_y<T, 12, true>;
-  e = opt_in(fy, ly << by);
-  if (e == cudaSuccess) e = opt_in(iy, ly << by);
-  if (e != cudaSuccess) return e;
   fy<<<gy * n_rhs, ty, ly << by, s>>>(spec, sstride, g.ax[1], g.K2, ycols, by, n_rhs, active, tw1);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
@@ -74,8 +84,6 @@ cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long
   const int bx = column_bits(lx, sizeof(C), xcols, n_rhs);
   const int gx = (xcols + (1 << bx) - 1) >> bx, tx = column_threads(g.ax[0], bx);
   const auto kx = max_radix(g.ax[0]) > 12 ? k_line_x<T, 16> : k_line_x<T, 12>;
-  e = opt_in(kx, lx << bx);
-  if (e != cudaSuccess) return e;
   kx<<<gx * n_rhs, tx, lx << bx, s>>>(spec, sstride, g.ax[0], xcols, bx, n_rhs, active, tw0, table);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
@@ -100,6 +108,7 @@ cudaError_t lines_green_table(T* table, const LineGrid& g, const void* const* ge
 }
 
 #define XFFT_LINES_INST(T)                                                                                         \
+  template cudaError_t lines_opt_in<T>();                                                                          \
   template cudaError_t lines_precondition<T>(const LineGrid&, T*, T*, void*, long long, long long, const int*,      \
                                              const void* const*, const T*, unsigned long long*, const T*,          \
                                              const RhsState*, double*, int, int, cudaStream_t);                    \
