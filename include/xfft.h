@@ -128,8 +128,13 @@ typedef struct {
                           without enrichment: each voxel takes the phase of its centre, where the
                           level set is the mean of its eight corner values (several level sets:
                           the first one negative there), and nX = 0 */
-  long long max_device_bytes; /* cap on the context's own device allocations (0 = none); a
-                          request above it fails with XFFT_ENOMEM as a failed cudaMalloc would */
+  long long max_device_bytes; /* cap on the context's device buffers (0 = none; small fixed tables of
+                          the grid and the FP32 plane passes' factors, 18 bytes per voxel on
+                          their grids, are outside it); a request above it fails with XFFT_ENOMEM as a
+                          failed cudaMalloc would.  The Green table of the line passes (36 bytes per
+                          voxel in FP64, 18 in FP32) and the reduced cut-tet records of FP64 contexts
+                          (1 KB per cut tet) count towards it and are given up when a call needs
+                          their room: the context then works without them, more slowly */
   long long spin_limit_ns; /* limit on the device time of one device-driven iteration loop (the
                           CG iterations between two residual checks run as one CUDA graph whose
                           while node repeats poll_every iterations until no right-hand side is

@@ -49,16 +49,16 @@ constexpr size_t kLoopStride = 64;
 constexpr size_t kLoopBytes = kLoopStride * kMaxBatch;
 
 struct xfft_ctx;
-static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes);
+static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool optional = false);
 static void dfree_bytes(xfft_ctx* c, void* p);
 
 // Device allocations of a context go through these two: they keep the context's byte count
 // (option max_device_bytes) and the size of every live block.
 template <typename T>
-static cudaError_t dalloc(xfft_ctx* c, T** p, size_t count) {
+static cudaError_t dalloc(xfft_ctx* c, T** p, size_t count, bool optional = false) {
   *p = nullptr;
   if (count == 0) count = 1;
-  return dalloc_bytes(c, (void**)p, count * sizeof(T));
+  return dalloc_bytes(c, (void**)p, count * sizeof(T), optional);
 }
 
 template <typename T>
@@ -121,6 +121,7 @@ struct xfft_ctx {
   double* eb64 = nullptr;
   float* eb32 = nullptr;
   FftPlan* fft = nullptr;
+  char* green = nullptr;  // the line passes' Green table in the solver's precision
   // solver workspace
   int cap_rhs = 0;
   long long cap_stride = 0;
@@ -191,7 +192,7 @@ struct Recycle {
   }
 };
 
-static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes) {
+static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool optional) {
   *p = nullptr;
   const size_t cap = (size_t)c->opt.max_device_bytes;
   if (c->recycling) {
@@ -228,13 +229,19 @@ static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes) {
         continue;
       }
     }
-    // the reduced element records are a speed-up that gives way to what a call cannot do without;
-    // nothing else holds their address (an apply captured by the caller does not read them)
-    if (e != cudaErrorMemoryAllocation || !c->cut_el) return e;
+    // the reduced element records and the Green table are speed-ups (optional) that give way to what
+    // a call cannot do without; nothing else holds their addresses (an apply captured by the caller does
+    // not read them)
+    if (optional || e != cudaErrorMemoryAllocation || (!c->cut_el && !c->green)) return e;
     cudaGetLastError();
     cudaStreamSynchronize(c->stream);
     drop_graphs(c);
-    dfree(c, c->cut_el);
+    if (c->cut_el) {
+      dfree(c, c->cut_el);
+    } else {
+      fft_table_drop(c->fft);
+      dfree(c, c->green);
+    }
   }
 }
 
@@ -409,7 +416,7 @@ extern "C" xfft_status xfft_create(xfft_ctx** out, const xfft_grid* grid, const 
   g.vol_tet = g.h[0] * g.h[1] * g.h[2] / 6.0;
   g.volY = grid->len[0] * grid->len[1] * grid->len[2];
   cudaError_t e = cudaSuccess;
-  c->fft = fft_plan_create(g, o.precision == XFFT_FP64, &e);
+  c->fft = fft_plan_create(g, o.precision == XFFT_FP32_REFINED, &e);
   if (!c->fft || e != cudaSuccess) {
     delete c;
     return fail(XFFT_ECUDA, std::string("FFT plan: ") + cudaGetErrorString(e));
@@ -429,6 +436,16 @@ extern "C" xfft_status xfft_create(xfft_ctx** out, const xfft_grid* grid, const 
   if ((e = cudaEventCreateWithFlags(&c->ev_join[0], cudaEventDisableTiming)) != cudaSuccess) {
     xfft_destroy(c);
     return fail(XFFT_ECUDA, cudaGetErrorString(e));
+  }
+  // the Green table, where it has room
+  const bool dbl = o.precision == XFFT_FP64;
+  if (const size_t bytes = fft_table_bytes(c->fft, dbl)) {
+    if (dalloc(c, &c->green, bytes, true) != cudaSuccess) {
+      cudaGetLastError();
+    } else if ((e = fft_table_fill(c->fft, dbl, c->green, c->stream)) != cudaSuccess) {
+      xfft_destroy(c);
+      return fail(XFFT_ECUDA, cudaGetErrorString(e));
+    }
   }
   *out = c;
   return XFFT_OK;
@@ -504,6 +521,7 @@ extern "C" void xfft_destroy(xfft_ctx* c) {
   if (c->stream) cudaStreamSynchronize(c->stream);
   free_micro(c);
   free_work(c);
+  dfree(c, c->green);
   fft_plan_destroy(c->fft);
   if (c->h_act) cudaFreeHost(c->h_act);
   if (c->h_st) cudaFreeHost(c->h_st);
@@ -674,7 +692,7 @@ extern "C" xfft_status xfft_set_microstructure_phases(xfft_ctx* c, int n_levelse
   if (c->opt.precision == XFFT_FP64 && c->ncut > 0) {
     // 1 KB per cut tet; where it does not fit (max_device_bytes, device memory) the FP64 applies run
     // on the moment records, with more arithmetic
-    const cudaError_t ea = dalloc(c, &c->cut_el, cut_el_reals(c->ncut));
+    const cudaError_t ea = dalloc(c, &c->cut_el, cut_el_reals(c->ncut), true);
     if (ea == cudaSuccess)
       CU(launch_cut_elements(cd, c->isD, c->nX, g, c->ph, c->has_scale ? c->scale : nullptr, c->cut_el, s));
     else
@@ -2001,7 +2019,7 @@ extern "C" xfft_status xfft_apply(xfft_ctx* c, int n_rhs, const double* d, const
 
 template <typename T>
 static xfft_status prec_entry(xfft_ctx* c, int n_rhs, const double* f, double* z, double* rr, int on_dev) {
-  CU(fft_plan_tables(c->fft, sizeof(T) == 8));
+  if (sizeof(T) == 4) CU(fft_plane_table(c->fft));
   const long long stride = stride_of(c);
   const size_t tot = (size_t)n_rhs * stride;
   double* scratch = nullptr;

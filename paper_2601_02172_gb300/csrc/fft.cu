@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "fft_lines.cuh"
@@ -36,7 +37,7 @@ struct FftPlan {
   float2* gsf[3];
   bool slab;               // the FP32 passes take the y-z plane path (fft_slab.cu)
   float* gtab = nullptr;   // its Green factor table
-  float* tabf = nullptr;   // Green tables of the line passes
+  float* tabf = nullptr;   // Green tables of the line passes, the caller's memory (fft_table_fill)
   double* tabd = nullptr;
   void* pool = nullptr;
 };
@@ -175,32 +176,61 @@ bool line_grid(LineGrid& lg, int n0, int n1, int n2, bool dbl) {
 
 static const void* const* as_void(const float2* const* p) { return reinterpret_cast<const void* const*>(p); }
 
-// The Green table of one precision, built once per plan (the solver's own precision at its creation,
-// the other one at the first step-level call that asks for it).
-cudaError_t fft_plan_tables(FftPlan* p, bool dbl) {
-  const GridDev& g = p->g;
-  const double ih[3] = {1.0 / g.h[0], 1.0 / g.h[1], 1.0 / g.h[2]};
-  const double hv = 0.5 * g.vol_tet;
-  const size_t n = 9 * (size_t)g.n0 * g.n1 * p->lf.K2;
-  cudaError_t e = cudaSuccess;
-  if (dbl) {
-    if (p->tabd) return cudaSuccess;
-    if ((e = cudaMalloc(&p->tabd, n * sizeof(double))) != cudaSuccess) return e;
-    e = lines_green_table<double>(p->tabd, p->ld, reinterpret_cast<const void* const*>(p->ged),
-                                  reinterpret_cast<const void* const*>(p->gsd), ih, hv, 0);
-  } else if (p->slab) {
-    if (p->gtab) return cudaSuccess;
-    if ((e = cudaMalloc(&p->gtab, slab_table_floats(g.n0, g.n1) * sizeof(float))) != cudaSuccess) return e;
-    e = slab_green_table(p->gtab, g.n0, g.n1, as_void(p->gef), as_void(p->gsf), ih, hv, 0);
-  } else {
-    if (p->tabf) return cudaSuccess;
-    if ((e = cudaMalloc(&p->tabf, n * sizeof(float))) != cudaSuccess) return e;
-    e = lines_green_table<float>(p->tabf, p->lf, as_void(p->gef), as_void(p->gsf), ih, hv, 0);
+template <typename T>
+static lines::SymbolArgs<T> symbol_args(const FftPlan* p) {
+  lines::SymbolArgs<T> sy;
+  for (int a = 0; a < 3; ++a) {
+    if constexpr (std::is_same<T, double>::value) {
+      sy.ge[a] = p->ged[a];
+      sy.gs[a] = p->gsd[a];
+    } else {
+      sy.ge[a] = p->gef[a];
+      sy.gs[a] = p->gsf[a];
+    }
+    sy.ih[a] = (T)(1.0 / p->g.h[a]);
   }
-  return e == cudaSuccess ? cudaDeviceSynchronize() : e;
+  sy.halfvol = (T)(0.5 * p->g.vol_tet);
+  sy.K2 = p->lf.K2;
+  return sy;
 }
 
-FftPlan* fft_plan_create(const GridDev& g, bool dbl, cudaError_t* err) {
+size_t fft_table_bytes(const FftPlan* p, bool dbl) {
+  if (!dbl && p->slab) return 0;
+  return 9 * (size_t)p->g.n0 * p->g.n1 * p->lf.K2 * (dbl ? sizeof(double) : sizeof(float));
+}
+
+cudaError_t fft_table_fill(FftPlan* p, bool dbl, void* mem, cudaStream_t s) {
+  const cudaError_t e = dbl ? lines_green_table<double>((double*)mem, p->ld, symbol_args<double>(p), s)
+                            : lines_green_table<float>((float*)mem, p->lf, symbol_args<float>(p), s);
+  if (e != cudaSuccess) return e;
+  if (dbl) p->tabd = (double*)mem;
+  else p->tabf = (float*)mem;
+  return cudaSuccess;
+}
+
+void fft_table_drop(FftPlan* p) {
+  p->tabf = nullptr;
+  p->tabd = nullptr;
+}
+
+cudaError_t fft_plane_table(FftPlan* p) {
+  if (!p->slab || p->gtab) return cudaSuccess;
+  const GridDev& g = p->g;
+  const double ih[3] = {1.0 / g.h[0], 1.0 / g.h[1], 1.0 / g.h[2]};
+  float* t = nullptr;
+  cudaError_t e = cudaMalloc(&t, slab_table_floats(g.n0, g.n1) * sizeof(float));
+  if (e != cudaSuccess) return e;
+  e = slab_green_table(t, g.n0, g.n1, as_void(p->gef), as_void(p->gsf), ih, 0.5 * g.vol_tet, 0);
+  if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  if (e != cudaSuccess) {
+    cudaFree(t);
+    return e;
+  }
+  p->gtab = t;
+  return cudaSuccess;
+}
+
+FftPlan* fft_plan_create(const GridDev& g, bool f32, cudaError_t* err) {
   *err = cudaSuccess;
   FftPlan* p = new FftPlan();
   p->g = g;
@@ -248,7 +278,7 @@ FftPlan* fft_plan_create(const GridDev& g, bool dbl, cudaError_t* err) {
   for (size_t i = 0; i < tot2d; ++i) hf[i] = make_float2((float)hd[i].x, (float)hd[i].y);
   *err = cudaMemcpy(dbase, hd.data(), tot2d * sizeof(double2), cudaMemcpyHostToDevice);
   if (*err == cudaSuccess) *err = cudaMemcpy(fbase, hf.data(), tot2d * sizeof(float2), cudaMemcpyHostToDevice);
-  if (*err == cudaSuccess) *err = fft_plan_tables(p, dbl);
+  if (*err == cudaSuccess && f32) *err = fft_plane_table(p);
   if (*err != cudaSuccess) {
     fft_plan_destroy(p);
     return nullptr;
@@ -260,8 +290,6 @@ void fft_plan_destroy(FftPlan* p) {
   if (!p) return;
   if (p->pool) cudaFree(p->pool);
   if (p->gtab) cudaFree(p->gtab);
-  if (p->tabf) cudaFree(p->tabf);
-  if (p->tabd) cudaFree(p->tabd);
   delete p;
 }
 
@@ -293,17 +321,15 @@ static cudaError_t standard_part(const FftPlan* p, float* f, float* z, void* spe
                              p->gtab, as_void(p->gef), as_void(p->gsf), ih, 0.5 * p->g.vol_tet, units, q, st, partials,
                              nparts, n_rhs, s);
   }
-  if (!p->tabf) return cudaErrorInvalidValue;
-  return lines_precondition<float>(p->lf, f, z, spec, stride, sstride, active, as_void(p->twf), p->tabf, units, q, st,
-                                   partials, nparts, n_rhs, s);
+  return lines_precondition<float>(p->lf, f, z, spec, stride, sstride, active, as_void(p->twf), p->tabf,
+                                   symbol_args<float>(p), units, q, st, partials, nparts, n_rhs, s);
 }
 static cudaError_t standard_part(const FftPlan* p, double* f, double* z, void* spec, long long stride,
                                  const int* active, double* partials, int nparts, int n_rhs, cudaStream_t s,
                                  unsigned long long* units, const double* q, const RhsState* st) {
-  if (!p->tabd) return cudaErrorInvalidValue;
   return lines_precondition<double>(p->ld, f, z, spec, stride, (long long)fft_spectrum_elems(p), active,
-                                    reinterpret_cast<const void* const*>(p->twd), p->tabd, units, q, st, partials,
-                                    nparts, n_rhs, s);
+                                    reinterpret_cast<const void* const*>(p->twd), p->tabd, symbol_args<double>(p),
+                                    units, q, st, partials, nparts, n_rhs, s);
 }
 
 template <typename T>

@@ -18,7 +18,8 @@
 // What bounds it: FP64, the FP64 pipe (2 FMAs per SM and clock); FP32, memory traffic: fields
 // and spectrum of one right-hand side are read and written once per pass.  The Green operator is a
 // table of the inverses (9 reals per frequency, built once per grid): its factorisation, about 200
-// operations and three square roots per frequency, costs more than the read.
+// operations and three square roots per frequency, costs more than the read.  Where a context has no
+// room for the table, pass 3 forms the factorisation instead.
 //
 // Per right-hand side inside the solvers (enriched block included), against Stockham passes with
 // compile-time plans where a length had one (256, 64) and run-time radix loops elsewhere:
@@ -185,12 +186,22 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR>())
 }
 
 // ---------------------------------------------------------------- x axis, Green operator, x inverse
-// columns q = j K2 + k2 of the n1 K2 lines of one component
-template <typename T, int MR>
+// What the symbol of a frequency is formed from (green_factor): e_a and e_a - 1 per axis, 1 / h_a, |T| / 2
+template <typename T>
+struct SymbolArgs {
+  const typename CplxOf<T>::type* ge[3];
+  const typename CplxOf<T>::type* gs[3];
+  T ih[3], halfvol;
+  int K2;
+};
+
+// columns q = j K2 + k2 of the n1 K2 lines of one component; TABLE: the inverses come from the table,
+// otherwise every frequency's symbol is factorised here
+template <typename T, int MR, bool TABLE>
 __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR, true>())
     k_line_x(typename CplxOf<T>::type* __restrict__ spec, long long sstride, LinePlan p, int cols, int lb, int n_rhs,
              const int* __restrict__ active, const typename CplxOf<T>::type* __restrict__ tw,
-             const T* __restrict__ table) {
+             const T* __restrict__ table, const SymbolArgs<T> sy) {
   typedef typename CplxOf<T>::type C;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int tile = blockIdx.x / n_rhs, rhs = blockIdx.x - tile * n_rhs;
@@ -247,7 +258,7 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR, true>())
         C* b = buf + ((w * R) << lb) + col;
         T g[9], h[9];  // the inverse at this frequency and (FP32) in flight the one at the next
         const T* t = table + (long long)k0 * cols + q;
-        if (kPipe == 2) {
+        if (TABLE && kPipe == 2) {
 #pragma unroll
           for (int i = 0; i < 9; ++i) g[i] = __ldg(t + i * cs);
         }
@@ -260,7 +271,25 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR, true>())
 #pragma unroll
           for (int r = 0; r < R; ++r) b[c * bc + (r << lb)] = v[r];
         }
-        for (int r = 0; r < R; ++r) {
+        if constexpr (!TABLE) {
+          const int j = q / sy.K2, k2 = q - j * sy.K2;
+#pragma unroll 1
+          for (int r = 0; r < R; ++r) {
+            const int kx = k0 + r * kstep;
+            C* f = b + (r << lb);
+            C F0 = f[0], F1 = f[bc], F2 = f[2 * bc];
+            fast::GreenFactor<C, T> gf;
+            if (fast::green_factor<C, T>(gf, sy.ge[0][kx], sy.ge[1][j], sy.ge[2][k2], sy.gs[0][kx], sy.gs[1][j],
+                                         sy.gs[2][k2], sy.ih[0], sy.ih[1], sy.ih[2], sy.halfvol))
+              fast::green_solve<C, T>(gf, F0, F1, F2);
+            else
+              F0 = F1 = F2 = zero;
+            f[0] = F0;
+            f[bc] = F1;
+            f[2 * bc] = F2;
+          }
+        }
+        for (int r = 0; TABLE && r < R; ++r) {
           if (kPipe == 1) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) g[i] = __ldg(t + i * cs);
@@ -608,20 +637,16 @@ __global__ void __launch_bounds__(kLineThreads, min_blocks<T, MR>())
 // Inverse of M(xi) per frequency: (00, 11, 22, Re 10, Im 10, Re 20, Im 20, Re 21, Im 21), each
 // [kx][j][k2]; zeros at xi = 0.  Formed from the Cholesky factor in the table's own precision.
 template <typename T>
-__global__ void k_line_green(T* __restrict__ table, int n0, int n1, int K2,
-                             const typename CplxOf<T>::type* __restrict__ ge0,
-                             const typename CplxOf<T>::type* __restrict__ ge1,
-                             const typename CplxOf<T>::type* __restrict__ ge2,
-                             const typename CplxOf<T>::type* __restrict__ gs0,
-                             const typename CplxOf<T>::type* __restrict__ gs1,
-                             const typename CplxOf<T>::type* __restrict__ gs2, T ih0, T ih1, T ih2, T halfvol) {
+__global__ void k_line_green(T* __restrict__ table, int n0, int n1, const SymbolArgs<T> sy) {
   typedef typename CplxOf<T>::type C;
+  const int K2 = sy.K2;
   const long long n = (long long)n0 * n1 * K2;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int k2 = (int)(i % K2), j = (int)((i / K2) % n1), kx = (int)(i / ((long long)K2 * n1));
     fast::GreenFactor<C, T> gf;
     T v[9] = {};
-    if (fast::green_factor<C, T>(gf, ge0[kx], ge1[j], ge2[k2], gs0[kx], gs1[j], gs2[k2], ih0, ih1, ih2, halfvol)) {
+    if (fast::green_factor<C, T>(gf, sy.ge[0][kx], sy.ge[1][j], sy.ge[2][k2], sy.gs[0][kx], sy.gs[1][j], sy.gs[2][k2],
+                                 sy.ih[0], sy.ih[1], sy.ih[2], sy.halfvol)) {
       C c[3];
 #pragma unroll
       for (int col = 0; col < 3; ++col) {
@@ -659,16 +684,16 @@ struct LineGrid {
 };
 bool line_grid(LineGrid& g, int n0, int n1, int n2, bool dbl);  // false for an unsupported length (fft.cu)
 
-// launchers of one precision (instantiated in fft_lines_f32.cu and fft_lines_f64.cu); lines_opt_in at the
+// launchers of one precision (table: nullptr where the context has none; instantiated in fft_lines_f32.cu and fft_lines_f64.cu); lines_opt_in at the
 // creation of a plan, for the current device
 template <typename T>
 cudaError_t lines_opt_in();
 template <typename T>
 cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec, long long stride, long long sstride,
-                               const int* active, const void* const* tw, const T* table, unsigned long long* units,
-                               const T* q, const RhsState* st, double* partials, int nparts, int n_rhs, cudaStream_t s);
+                               const int* active, const void* const* tw, const T* table,
+                               const lines::SymbolArgs<T>& sy, unsigned long long* units, const T* q,
+                               const RhsState* st, double* partials, int nparts, int n_rhs, cudaStream_t s);
 template <typename T>
-cudaError_t lines_green_table(T* table, const LineGrid& g, const void* const* ge, const void* const* gs,
-                              const double* ih, double halfvol, cudaStream_t s);
+cudaError_t lines_green_table(T* table, const LineGrid& g, const lines::SymbolArgs<T>& sy, cudaStream_t s);
 
 }  // namespace xfft

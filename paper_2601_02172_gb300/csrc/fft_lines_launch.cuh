@@ -37,8 +37,8 @@ cudaError_t lines_opt_in() {
   const void* const kernels[] = {
       (const void*)k_line_z_fwd<T, 12>,    (const void*)k_line_z_fwd<T, 16>,    (const void*)k_line_z_inv<T, 12>,
       (const void*)k_line_z_inv<T, 16>,    (const void*)k_line_y<T, 12, false>, (const void*)k_line_y<T, 16, false>,
-      (const void*)k_line_y<T, 12, true>,  (const void*)k_line_y<T, 16, true>,  (const void*)k_line_x<T, 12>,
-      (const void*)k_line_x<T, 16>};
+      (const void*)k_line_y<T, 12, true>,  (const void*)k_line_y<T, 16, true>,  (const void*)k_line_x<T, 12, true>,
+      (const void*)k_line_x<T, 16, true>,  (const void*)k_line_x<T, 12, false>, (const void*)k_line_x<T, 16, false>};
   for (const void* k : kernels) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineShared);
     if (e != cudaSuccess) return e;
@@ -48,9 +48,9 @@ cudaError_t lines_opt_in() {
 
 template <typename T>
 cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long long stride, long long sstride,
-                               const int* active, const void* const* tw, const T* table, unsigned long long* units,
-                               const T* q, const RhsState* st, double* partials, int nparts, int n_rhs,
-                               cudaStream_t s) {
+                               const int* active, const void* const* tw, const T* table,
+                               const lines::SymbolArgs<T>& sy, unsigned long long* units, const T* q,
+                               const RhsState* st, double* partials, int nparts, int n_rhs, cudaStream_t s) {
   using namespace lines;
   typedef typename CplxOf<T>::type C;
   C* spec = static_cast<C*>(spec_v);
@@ -83,8 +83,10 @@ cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long
   const size_t lx = 3 * sizeof(C) * g.n0;
   const int bx = column_bits(lx, sizeof(C), xcols, n_rhs);
   const int gx = (xcols + (1 << bx) - 1) >> bx, tx = column_threads(g.ax[0], bx);
-  const auto kx = max_radix(g.ax[0]) > 12 ? k_line_x<T, 16> : k_line_x<T, 12>;
-  kx<<<gx * n_rhs, tx, lx << bx, s>>>(spec, sstride, g.ax[0], xcols, bx, n_rhs, active, tw0, table);
+  const bool big_x = max_radix(g.ax[0]) > 12;
+  const auto kx = table ? (big_x ? k_line_x<T, 16, true> : k_line_x<T, 12, true>)
+                        : (big_x ? k_line_x<T, 16, false> : k_line_x<T, 12, false>);
+  kx<<<gx * n_rhs, tx, lx << bx, s>>>(spec, sstride, g.ax[0], xcols, bx, n_rhs, active, tw0, table, sy);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   iy<<<gy * n_rhs, ty, ly << by, s>>>(spec, sstride, g.ax[1], g.K2, ycols, by, n_rhs, active, tw1);
@@ -96,23 +98,19 @@ cudaError_t lines_precondition(const LineGrid& g, T* f, T* z, void* spec_v, long
 }
 
 template <typename T>
-cudaError_t lines_green_table(T* table, const LineGrid& g, const void* const* ge, const void* const* gs,
-                              const double* ih, double halfvol, cudaStream_t s) {
-  typedef typename lines::CplxOf<T>::type C;
+cudaError_t lines_green_table(T* table, const LineGrid& g, const lines::SymbolArgs<T>& sy, cudaStream_t s) {
   const long long n = (long long)g.n0 * g.n1 * g.K2;
   const int blocks = (int)std::min<long long>((n + 127) / 128, 152 * 64);
-  lines::k_line_green<T><<<blocks, 128, 0, s>>>(table, g.n0, g.n1, g.K2, (const C*)ge[0], (const C*)ge[1],
-                                                (const C*)ge[2], (const C*)gs[0], (const C*)gs[1], (const C*)gs[2],
-                                                (T)ih[0], (T)ih[1], (T)ih[2], (T)halfvol);
+  lines::k_line_green<T><<<blocks, 128, 0, s>>>(table, g.n0, g.n1, sy);
   return cudaGetLastError();
 }
 
 #define XFFT_LINES_INST(T)                                                                                         \
   template cudaError_t lines_opt_in<T>();                                                                          \
   template cudaError_t lines_precondition<T>(const LineGrid&, T*, T*, void*, long long, long long, const int*,      \
-                                             const void* const*, const T*, unsigned long long*, const T*,          \
-                                             const RhsState*, double*, int, int, cudaStream_t);                    \
-  template cudaError_t lines_green_table<T>(T*, const LineGrid&, const void* const*, const void* const*,           \
-                                            const double*, double, cudaStream_t);
+                                             const void* const*, const T*, const lines::SymbolArgs<T>&,            \
+                                             unsigned long long*, const T*, const RhsState*, double*, int, int,    \
+                                             cudaStream_t);                                                        \
+  template cudaError_t lines_green_table<T>(T*, const LineGrid&, const lines::SymbolArgs<T>&, cudaStream_t);
 
 }  // namespace xfft

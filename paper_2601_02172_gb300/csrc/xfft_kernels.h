@@ -158,9 +158,15 @@ cudaError_t launch_voxel_stress(const double* u, const double* isD, CutData cd,
 
 // ---- preconditioner (fft.cu)
 struct FftPlan;  // opaque
-// the plan with the Green table of one precision (dbl: FP64); fft_plan_tables adds another's
-FftPlan* fft_plan_create(const GridDev& g, bool dbl, cudaError_t* err);
-cudaError_t fft_plan_tables(FftPlan* p, bool dbl);
+// f32: with the factor table that the FP32 y-z plane passes need (fft_plane_table adds it later)
+FftPlan* fft_plan_create(const GridDev& g, bool f32, cudaError_t* err);
+cudaError_t fft_plane_table(FftPlan* p);
+// The line passes' Green table of one precision, a speed-up in memory of the caller: its size (0: the
+// plane passes serve this precision), its filling on a stream (used from then on), and its end (the
+// passes form the symbols themselves).
+size_t fft_table_bytes(const FftPlan* p, bool dbl);
+cudaError_t fft_table_fill(FftPlan* p, bool dbl, void* mem, cudaStream_t s);
+void fft_table_drop(FftPlan* p);
 void fft_plan_destroy(FftPlan* p);
 size_t fft_spectrum_elems(const FftPlan* p);  // complex elements per RHS
 // z = P^-1 f per RHS (std part via FFT + Green, enr part identity); f^T z partials into

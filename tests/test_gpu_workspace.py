@@ -138,3 +138,75 @@ def test_captured_apply_outlives_the_reduced_records(xf):
         del junk, graph
         s.close()
     assert served >= 4 and refused >= 1
+
+
+def test_green_table_is_counted_and_gives_way(xf):
+    """The line passes' Green table (9 reals per frequency) counts towards max_device_bytes and is only taken
+    where it fits: a context whose cap is below its size holds next to nothing, and over caps from the smallest
+    that a preconditioner call fits in, a quarter of the table apart, the results are those without
+    a cap (1e-11 and 2e-5 of their norm for the other way of forming the inverses)."""
+    import torch
+    n = (90, 60, 50)
+    table = 9 * n[0] * n[1] * (n[2] // 2 + 1)
+    L = synth.sphere_levelset(n, (0.5, 0.45, 0.55), 0.3)
+    for precision, size, tol in (("fp64", 8 * table, 1e-11), ("fp32", 4 * table, 2e-5)):
+        s = xf.Solver(n, precision=precision)
+        torch.cuda.synchronize()
+        free0, _ = torch.cuda.mem_get_info()
+        capped = [xf.Solver(n, precision=precision, max_device_bytes=size - 1) for _ in range(4)]
+        torch.cuda.synchronize()
+        assert free0 - torch.cuda.mem_get_info()[0] < 4 * size - (2 << 20)
+        for c in capped:
+            c.close()
+        s.set_microstructure(L, LM, LP)
+        f = np.random.default_rng(4).normal(size=(2, s.stride))
+        for c in range(3):
+            f[:, c * s.N:(c + 1) * s.N] -= f[:, c * s.N:(c + 1) * s.N].mean(1, keepdims=True)
+        ref, rr = s.precondition(f, precision=precision)
+        C0 = s.effective_stiffness()[0]
+        s.close()
+
+        def serves(cap):
+            s = xf.Solver(n, precision=precision, max_device_bytes=cap)
+            try:
+                s.set_microstructure(L, LM, LP)
+                z, zr = s.precondition(f, precision=precision)
+                assert _rel(z, ref) < tol and _rel(zr, rr) < 10 * tol
+                return True
+            except xf.XfftError as e:
+                assert e.status == xf.capi.XFFT_ENOMEM
+                return False
+            finally:
+                s.close()
+
+        low, high = 0, 1 << 30
+        while high - low > size // 4:
+            mid = (low + high) // 2
+            low, high = (low, mid) if serves(mid) else (mid, high)
+        assert all(serves(high + k * (size // 4)) for k in range(7))
+        s = xf.Solver(n, precision=precision, max_device_bytes=1 << 30)
+        s.set_microstructure(L, LM, LP)
+        assert _rel(s.effective_stiffness()[0], C0) < 1e-9
+        s.close()
+
+
+@pytest.mark.parametrize("n", [(16, 18, 20), (30, 12, 10), (150, 8, 6), (256, 6, 4)])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_symbols_formed_in_the_pass(xf, n, precision):
+    """A context has the Green table of its own precision; a preconditioner call in the other one forms the
+    symbols in the pass.  Both against the oracle (1e-11 and 2e-5 of the norm) for each class of x lengths."""
+    from oracle import XFEM
+    ell = (1.0, 1.2, 0.9)
+    L = np.ones(n)
+    L[1, 2, 3] = -0.7
+    s = xf.Solver(n, ell, precision=precision)
+    s.set_microstructure(L, LM, LP)
+    o = XFEM(L, n, ell, lame_minus=LM, lame_plus=LP)
+    f = np.random.default_rng(6).normal(size=(2, s.stride))
+    for c in range(3):
+        f[:, c * s.N:(c + 1) * s.N] -= f[:, c * s.N:(c + 1) * s.N].mean(1, keepdims=True)
+    for prec, tol in (("fp64", 1e-11), ("fp32", 2e-5)):
+        z, _ = s.precondition(f, precision=prec)
+        for k in range(2):
+            assert _rel(z[k], o.precondition(f[k], green="fft")) < tol, prec
+    s.close()
