@@ -181,25 +181,34 @@ static void free_spare(xfft_ctx* c) {
 // A call that replaces buffers (a new microstructure, another workspace) hands the blocks it frees to
 // the allocations that follow: the context's work is ordered on its stream, so a block can be reused
 // at once, and twenty cudaMalloc / cudaFree pairs (2.5 ms of a 5.7 ms set-up at 128^3) fall away.
-// What the scope did not use is freed at its end.  With a cap on the device bytes every block has its
-// exact size and is freed as before.
+// What the scope did not use is freed at its end.  A reused block is at most a sixteenth larger than
+// what it serves, and blocks that replace others are taken that much larger, for the next, slightly
+// different microstructure.  Where bytes matter (a cap on them, or less than half of the device's memory
+// free), and for a context's first blocks, every block has its exact size and is freed as before: what a
+// single use of the context fits in is not taken by spare room.
 struct Recycle {
   xfft_ctx* c;
-  explicit Recycle(xfft_ctx* c_) : c(c_) { c->recycling = c->opt.max_device_bytes == 0; }
+  Recycle(xfft_ctx* c_, bool replaces) : c(c_) {
+    size_t free = 0, total = 0;
+    c->recycling = replaces && c->opt.max_device_bytes == 0 && cudaMemGetInfo(&free, &total) == cudaSuccess &&
+                   free > total / 2;
+  }
   ~Recycle() {
     c->recycling = false;
     free_spare(c);
   }
 };
 
+static size_t block_slack(size_t bytes) { return bytes / 16; }
+
 static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool optional) {
   *p = nullptr;
   const size_t cap = (size_t)c->opt.max_device_bytes;
   if (c->recycling) {
-    // the smallest spare block that holds the request without wasting a quarter of itself
+    // the smallest spare block that holds the request
     int best = -1;
     for (int i = 0; i < (int)c->spare.size(); ++i)
-      if (c->spare[i].second >= bytes && c->spare[i].second <= bytes + bytes / 3 + 4096 &&
+      if (c->spare[i].second >= bytes && c->spare[i].second <= bytes + block_slack(bytes) + 4096 &&
           (best < 0 || c->spare[i].second < c->spare[best].second))
         best = i;
     if (best >= 0) {
@@ -213,8 +222,7 @@ static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool option
   for (;;) {
     cudaError_t e = cudaErrorMemoryAllocation;
     if (cap == 0 || c->bytes + bytes <= cap) {
-      // a sixteenth of slack lets the next microstructure's slightly larger lists reuse the block
-      const size_t want = c->recycling ? bytes + bytes / 16 : bytes;
+      const size_t want = c->recycling ? bytes + block_slack(bytes) : bytes;
       e = cudaMalloc(p, want);
       if (e == cudaSuccess) {
         c->blocks[*p] = want;
@@ -574,7 +582,7 @@ extern "C" xfft_status xfft_set_microstructure_phases(xfft_ctx* c, int n_levelse
   for (int p = 0; p < nph; ++p)
     if (!(lame[2 * p + 1] > 0.0) || !(3.0 * lame[2 * p] + 2.0 * lame[2 * p + 1] > 0.0))
       return fail(XFFT_EINVAL, "Lame constants must give a positive definite stiffness");
-  Recycle recycle(c);
+  Recycle recycle(c, c->Ls != nullptr);
   free_micro(c);
   const GridDev& g = c->g;
   const long long N = g.N;
@@ -776,7 +784,7 @@ static xfft_status ensure_work(xfft_ctx* c, int n_rhs, int prec) {
     c->partials_count = need;
     return XFFT_OK;
   }
-  Recycle recycle(c);
+  Recycle recycle(c, c->cap_rhs > 0);
   free_work(c);
   const size_t tot = (size_t)n_rhs * stride;
   if (prec == XFFT_FP64) {

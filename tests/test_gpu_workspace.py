@@ -210,3 +210,30 @@ def test_symbols_formed_in_the_pass(xf, n, precision):
         for k in range(2):
             assert _rel(z[k], o.precondition(f[k], green="fft")) < tol, prec
     s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+def test_first_blocks_have_their_exact_size(xf, precision):
+    """A context without a cap takes no more device memory for its first microstructure and solve than one
+    with a cap that it stays below, and after a second, smaller microstructure no more than a sixteenth above
+    (the driver hands out 2 MB pieces: 24 MB of tolerance for some fifty blocks of a gigabyte)."""
+    import torch
+    n = (96, 96, 96)
+    big, small = (np.minimum(synth.sphere_levelset(n, (0.3, 0.3, 0.3), r), synth.sphere_levelset(n, (0.8, 0.8, 0.8), r))
+                  for r in (0.2, 0.18))
+    used = []
+    for cap in (1 << 34, 0):
+        torch.cuda.synchronize()
+        free0, _ = torch.cuda.mem_get_info()
+        s = xf.Solver(n, precision=precision, max_device_bytes=cap, autotune=False, tol=1e-4)
+        use = []
+        for L in (big, small):
+            s.set_microstructure(L, LM, LP)
+            assert s.effective_stiffness()[1]["converged"]
+            torch.cuda.synchronize()
+            use.append(free0 - torch.cuda.mem_get_info()[0])
+        used.append(use)
+        s.close()
+    (e1, e2), (r1, r2) = used
+    assert r1 <= e1 + (24 << 20), used
+    assert r2 <= e2 * 17 / 16 + (24 << 20), used
