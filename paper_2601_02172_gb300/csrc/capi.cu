@@ -163,6 +163,7 @@ struct xfft_ctx {
   // blocks freed inside a Recycle scope, for the allocations that follow in it
   std::vector<std::pair<void*, size_t>> spare;
   bool recycling = false;
+  int roomy = -1;
   // Euclidean Barzilai-Borwein steps: <d, d>, <A d, A d> partial sums
   double* bbpart = nullptr;
   // launch shapes picked by the tuner (0: defaults): the FP32 cut-tet kernel's grid and
@@ -181,17 +182,17 @@ static void free_spare(xfft_ctx* c) {
 // A call that replaces buffers (a new microstructure, another workspace) hands the blocks it frees to
 // the allocations that follow: the context's work is ordered on its stream, so a block can be reused
 // at once, and twenty cudaMalloc / cudaFree pairs (2.5 ms of a 5.7 ms set-up at 128^3) fall away.
-// What the scope did not use is freed at its end.  A reused block is at most a sixteenth larger than
-// what it serves, and blocks that replace others are taken that much larger, for the next, slightly
-// different microstructure.  Where bytes matter (a cap on them, or less than half of the device's memory
-// free), and for a context's first blocks, every block has its exact size and is freed as before: what a
-// single use of the context fits in is not taken by spare room.
+// What the scope did not use is freed at its end.  While more than half of the device's memory is free, a
+// reused block may be a third larger than what it serves and blocks that replace others are taken a
+// sixteenth larger, for the next, slightly different microstructure (128^3, changing radii: 1.1 ms instead
+// of 1.5 with a sixteenth for both).  Otherwise, and for a context's first blocks, every block has its exact
+// size, so that what a single use of the context fits in is not taken by spare room.  With a cap on the
+// bytes nothing is recycled.
 struct Recycle {
   xfft_ctx* c;
   Recycle(xfft_ctx* c_, bool replaces) : c(c_) {
-    size_t free = 0, total = 0;
-    c->recycling = replaces && c->opt.max_device_bytes == 0 && cudaMemGetInfo(&free, &total) == cudaSuccess &&
-                   free > total / 2;
+    c->recycling = replaces && c->opt.max_device_bytes == 0;
+    c->roomy = -1;
   }
   ~Recycle() {
     c->recycling = false;
@@ -199,19 +200,28 @@ struct Recycle {
   }
 };
 
-static size_t block_slack(size_t bytes) { return bytes / 16; }
+// whether a block of this many bytes may have spare room; the device is asked once per scope, and not for
+// blocks below a megabyte
+static bool roomy(xfft_ctx* c, size_t bytes) {
+  if (bytes < (1u << 20)) return true;
+  if (c->roomy < 0) {
+    size_t free = 0, total = 0;
+    c->roomy = cudaMemGetInfo(&free, &total) == cudaSuccess && free > total / 2;
+  }
+  return c->roomy != 0;
+}
 
 static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool optional) {
   *p = nullptr;
   const size_t cap = (size_t)c->opt.max_device_bytes;
   if (c->recycling) {
-    // the smallest spare block that holds the request
+    // the smallest spare block that holds the request without wasting a quarter of itself
     int best = -1;
     for (int i = 0; i < (int)c->spare.size(); ++i)
-      if (c->spare[i].second >= bytes && c->spare[i].second <= bytes + block_slack(bytes) + 4096 &&
+      if (c->spare[i].second >= bytes && c->spare[i].second <= bytes + bytes / 3 + 4096 &&
           (best < 0 || c->spare[i].second < c->spare[best].second))
         best = i;
-    if (best >= 0) {
+    if (best >= 0 && (c->spare[best].second == bytes || roomy(c, bytes))) {
       *p = c->spare[best].first;
       c->blocks[*p] = c->spare[best].second;
       c->bytes += c->spare[best].second;
@@ -222,7 +232,7 @@ static cudaError_t dalloc_bytes(xfft_ctx* c, void** p, size_t bytes, bool option
   for (;;) {
     cudaError_t e = cudaErrorMemoryAllocation;
     if (cap == 0 || c->bytes + bytes <= cap) {
-      const size_t want = c->recycling ? bytes + block_slack(bytes) : bytes;
+      const size_t want = c->recycling && roomy(c, bytes) ? bytes + bytes / 16 : bytes;
       e = cudaMalloc(p, want);
       if (e == cudaSuccess) {
         c->blocks[*p] = want;
