@@ -18,6 +18,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 #include <vector>
 
@@ -230,6 +231,20 @@ cudaError_t fft_plane_table(FftPlan* p) {
   return cudaSuccess;
 }
 
+// the line kernels' shared-memory opt-in, once per device (20 calls of 10-20 us)
+static cudaError_t opt_in_device() {
+  static std::mutex mu;
+  static std::vector<int> done;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  if (std::find(done.begin(), done.end(), dev) != done.end()) return cudaSuccess;
+  if ((e = lines_opt_in<float>()) == cudaSuccess) e = lines_opt_in<double>();
+  if (e == cudaSuccess) done.push_back(dev);
+  return e;
+}
+
 FftPlan* fft_plan_create(const GridDev& g, bool f32, cudaError_t* err) {
   *err = cudaSuccess;
   FftPlan* p = new FftPlan();
@@ -240,7 +255,7 @@ FftPlan* fft_plan_create(const GridDev& g, bool f32, cudaError_t* err) {
     delete p;
     return nullptr;
   }
-  if ((*err = lines_opt_in<float>()) != cudaSuccess || (*err = lines_opt_in<double>()) != cudaSuccess) {
+  if ((*err = opt_in_device()) != cudaSuccess) {
     delete p;
     return nullptr;
   }

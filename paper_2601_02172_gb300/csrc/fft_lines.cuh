@@ -6,7 +6,8 @@
 //   pass 4  y axis inverse    pass 5  z axis complex to real, fused f^T z partial sums
 // Spectrum layout per right-hand side: [c][i][j][k2], k2 <= n2 / 2 contiguous, twice the transform.
 //
-// A length n = R1 RM RL (RM = 1 where two factors of at most 25 do) is transformed by decimation
+// A length n = R1 RM RL (factors of at most 16, RM = 1 where two are the better choice: line_plan in
+// fft.cu) is transformed by decimation
 // in time in place: index (n1, m, l) = n1 RM RL + m RL + l; an R1-point DFT over n1 for every
 // (m, l), twiddle W_n^(k1 (m RL + l)); an RM-point DFT over m, twiddle W_(RM RL)^(km l); an RL-point
 // DFT over l; frequency k = k1 + R1 km + R1 RM kl.  The first DFT reads its inputs from global
@@ -19,7 +20,8 @@
 // and spectrum of one right-hand side are read and written once per pass.  The Green operator is a
 // table of the inverses (9 reals per frequency, built once per grid): its factorisation, about 200
 // operations and three square roots per frequency, costs more than the read.  Where a context has no
-// room for the table, pass 3 forms the factorisation instead.
+// room for the table, pass 3 forms the factorisation instead (whole call, with and without the table:
+// FP64 256^3 8.3 and 12.0 ms, FP32 0.61 and 0.67 ms).
 //
 // Per right-hand side inside the solvers (enriched block included), against Stockham passes with
 // compile-time plans where a length had one (256, 64) and run-time radix loops elsewhere:
@@ -684,8 +686,8 @@ struct LineGrid {
 };
 bool line_grid(LineGrid& g, int n0, int n1, int n2, bool dbl);  // false for an unsupported length (fft.cu)
 
-// launchers of one precision (table: nullptr where the context has none; instantiated in fft_lines_f32.cu and fft_lines_f64.cu); lines_opt_in at the
-// creation of a plan, for the current device
+// launchers of one precision (instantiated in fft_lines_f32.cu and fft_lines_f64.cu; table: nullptr where
+// the context has none); lines_opt_in for the current device before the first launch
 template <typename T>
 cudaError_t lines_opt_in();
 template <typename T>

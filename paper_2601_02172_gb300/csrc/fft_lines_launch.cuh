@@ -29,7 +29,7 @@ inline int max_radix(const LinePlan& p) { return std::max(p.R1, std::max(p.RM, p
 }  // namespace lines
 
 // All lengths share the kernels of a precision and radix class, and the opt-in to more than 48 KB of
-// shared memory belongs to the kernel, not to a launch: every plan gives the same, largest one, so that
+// shared memory belongs to the kernel, not to a launch: it is given once, at its largest, so that
 // no launch of another grid (another context in another thread, another node of a graph) finds it lowered.
 template <typename T>
 cudaError_t lines_opt_in() {
