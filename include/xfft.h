@@ -259,6 +259,9 @@ xfft_status xfft_grad_phases(xfft_ctx* ctx, const double dL_dCeff[36], double* d
  *   xfft_precondition: z = P^{-1} f with P = diag(A0_11, I) (eqs. scaledPreconditioner,
  *                      GreenHermitian); the standard part of f must have zero mean per
  *                      component.  rr (n_rhs, host, may be NULL) receives f^T z.
+ * q is summed with atomic additions where tets are cut and, in FP64 and double-word arithmetic, at the
+ * nodes between the stencil's tiles: two calls on the same input may differ in the last places.
+ * <d, A d> and the stress integrals of fixed launch shapes are summed in a fixed order of blocks.
  * precision: XFFT_FP64, XFFT_FP32_REFINED (= 1, the FP32 kernels) or XFFT_DW (xfft_apply only:
  * double-word kernels); inputs and outputs stay double.  Other values: XFFT_EINVAL. */
 xfft_status xfft_apply(xfft_ctx* ctx, int n_rhs, const double* d, const double* eps_bar,
@@ -301,12 +304,12 @@ xfft_status xfft_profile_read(xfft_ctx* ctx, double ms[16], long long launches[1
  *            int_Y C grad^s d (Mandel 6) per RHS.
  * Its reduction scratch is a fixed array in the library's device memory (about 1.8 MB,
  * present on every GPU that loads the library until the process exits), so it serves at most
- * XFFT_NOALLOC_MAX_RHS right-hand sides and grids whose apply launches at most
- * XFFT_NOALLOC_MAX_PARTS blocks, each writing one partial sum per value: the stencil's
- * ceil(n2 / 15) ceil(n1 / 15) ceil(n0 / 32) blocks plus the cut-tet kernel's blocks (at most
- * a few waves of the GPU's SMs).  With the default tiling 256^3 grids fit and 384^3 grids do
- * not; larger requests return XFFT_EINVAL and touch nothing.  The scratch address of a device
- * is looked up once, by the first xfft_set_microstructure (or xfft_apply_noalloc) on that
+ * XFFT_NOALLOC_MAX_RHS right-hand sides and grids of at most XFFT_NOALLOC_MAX_PARTS blocks, by a
+ * fixed rule: ceil(n2 / 15) ceil(n1 / 15) ceil(n0 / 32) blocks of voxels plus one per 128 cut tets,
+ * at most 1216.  256^3 grids fit and 384^3 grids do not; larger requests return XFFT_EINVAL and
+ * touch nothing.  (The FP64 kernels launch at most 1216 and 2432 blocks per right-hand side, each
+ * writing one partial sum per value; the rule is the interface's, not theirs.)  The scratch address
+ * of a device is looked up once, by the first xfft_set_microstructure (or xfft_apply_noalloc) on that
  * device; a first lookup attempted while the context's stream is being captured returns
  * XFFT_ESTATE instead.
  * The call may be captured into a CUDA graph; the graph reads the microstructure's buffers and can

@@ -24,8 +24,8 @@ int apply_uncut_blocks(const GridDev& g) {
 
 // Tile of the FP64 / double-word stencil.  The kernel is bound by the arithmetic pipe of its SMs,
 // so its time is about the operations of the busiest SM, in warp instructions: 210 per plane and
-// warp of voxels, 22 per plane and 32 of the tile's (ty + 1)(tz + 1) nodes (update, force sums), one
-// more node plane per item.  Items are cut small enough to spread evenly (a grid of 16^3 voxels is
+// warp of voxels, 22 per plane and 32 of the tile's (ty + 1)(tz + 1) nodes (update, force sums; an estimate,
+// the sums for a caller add three per node), one more node plane per item.  Items are cut small enough to spread evenly (a grid of 16^3 voxels is
 // 128 warps, one per SM); fewer than about four warps per SM leave the pipe waiting for its own
 // results.  Every tile shape that fills the block (equal parts of a row, as many rows as fit) and
 // power-of-two plane counts are compared by that estimate.

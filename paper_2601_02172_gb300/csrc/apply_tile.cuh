@@ -17,7 +17,8 @@
 //    error grows with the mean of d (10^6 times its variation: 4e-11 of the result on 48^3), that of the
 //    tets' energies does not, and the relative sum matches those at 3 subtractions per node instead of 36
 //    multiply-adds per voxel.  The CG directions (FUSED) have no mean.
-// About 230 operations per voxel (uniform voxels) instead of about 470, and no padding of the
+// About 240 operations per voxel (uniform voxels: 210 for the voxel, 22 for each of its about 1.3 node
+// visits; counted by ncu at 64^3: 246 with the caller's sums) instead of about 470, and no padding of the
 // plane to 15 x 15 node tiles: the tile's shape is a launch parameter (pick_tile).
 #pragma once
 
